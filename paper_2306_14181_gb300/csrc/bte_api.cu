@@ -16,6 +16,7 @@
 #include "../../include/bte.h"
 #include "bte_internal.h"
 #include "bte_tiled.h"
+#include "bte_stream.h"
 #include "bte_adjoint.h"
 
 using namespace bte;
@@ -68,6 +69,9 @@ struct bte_ctx {
     // tiled-kernel plan
     TiledPlan plan;
     bool tiled = false;
+    // register-streaming plan of the grids the tiled kernel does not take
+    StreamPlan splan;
+    bool streamed = false;
     // persistent single-CTA path (small 1-D FP32 problems): per-call source amplitudes
     bool persist = false;
     float *d_amp = nullptr;
@@ -373,6 +377,7 @@ static void free_all(bte_ctx *c) {
     for (void *p : ptrs)
         if (p) cudaFree(p);
     tiled_free(c->plan);
+    stream_free(c->splan);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
     c->ev.clear();
     if (c->h_src) cudaFreeHost(c->h_src);
@@ -551,6 +556,11 @@ extern "C" bte_status bte_create(const bte_grid *grid, const bte_bands *bands, c
             return bail(BTE_EUNSUPPORTED);
         }
     }
+    if (!c->persist && !c->tiled) {
+        std::string why;  // not applicable: the generic kernel
+        c->streamed = stream_plan(c->dim, c->n, c->nb, c->nd, c->s.data(), c->bc, c->jump, c->storage, c->limiter,
+                                  c->splan, why);
+    }
     // wall-cell slots (a multiple of 8 elements keeps every e_diff row 16-byte aligned)
     c->wc_max = 1;
     for (int a = 0; a < c->dim; ++a) {
@@ -620,6 +630,7 @@ extern "C" bte_status bte_create(const bte_grid *grid, const bte_bands *bands, c
         // moment partials: band-major rows for the generic passes, segment rows for the tiled one
         size_t np = (size_t)c->nb * c->ncell;
         if (c->tiled) np = std::max(np, (size_t)c->plan.G * c->plan.tcells);
+        if (c->streamed) np *= c->splan.nchunk;  // a row per part of a band's directions
         if ((st = dalloc(c, &c->P, np)) != BTE_OK) return bail(st);
     }
     for (int i = 0; i < 2; ++i)
@@ -662,6 +673,13 @@ extern "C" bte_status bte_create(const bte_grid *grid, const bte_bands *bands, c
         std::string why;
         if (!tiled_setup(c->plan, make_args(c), why)) {
             c->err = "tiled kernel setup failed: " + why;
+            return bail(BTE_ECUDA);
+        }
+    }
+    if (c->streamed) {
+        std::string why;
+        if (!stream_setup(c->splan, why)) {
+            c->err = "streaming kernel setup failed: " + why;
             return bail(BTE_ECUDA);
         }
     }
@@ -921,6 +939,17 @@ extern "C" bte_status bte_interface(bte_ctx *a, int wa, bte_ctx *b, int wb, cons
     return iface_mix(a);
 }
 
+// The forward step's main kernel by the context's plan.
+static cudaError_t launch_forward(bte_ctx *c, const StepArgs &a, cudaStream_t strm) {
+    if (c->tiled) {
+        const cudaError_t e = launch_step_tiled(a, c->plan, strm);
+        c->plan.stall = 0;
+        return e;
+    }
+    if (c->streamed) return launch_step_stream(a, c->splan, strm);
+    return launch_step_generic(a, c->storage, c->limiter, strm);
+}
+
 static bte_status step_one(bte_ctx *c, cudaStream_t strm) {
     {
         StepArgs a = make_args(c);
@@ -937,18 +966,14 @@ static bte_status step_one(bte_ctx *c, cudaStream_t strm) {
         cudaError_t e;
         cudaEvent_t ev;
         if (c->prof) TRY(prof_event(c, &ev));
-        if (c->tiled) {
-            e = launch_step_tiled(a, c->plan, strm);
-            c->plan.stall = 0;
-        } else {
-            e = launch_step_generic(a, c->storage, c->limiter, strm);
-        }
+        e = launch_forward(c, a, strm);
         if (e != cudaSuccess) return fail(c, BTE_ECUDA, "forward step launch: %s", cudaGetErrorString(e));
         if (c->prof) TRY(prof_event(c, &ev));
         // T_L^{n+1} goes to the buffer of the old code reference; T_L^n becomes the reference of
         // the new state
         float *TL_next = c->R;
         if (c->tiled) e = launch_finalize_tiled(a, c->plan, c->storage, TL_next, strm);
+        else if (c->streamed) e = launch_finalize_stream(a, c->splan, TL_next, strm);
         else e = launch_finalize(a, c->G, TL_next, strm);
         if (e != cudaSuccess) return fail(c, BTE_ECUDA, "finalize launch: %s", cudaGetErrorString(e));
         if (c->prof) TRY(prof_event(c, &ev));
@@ -1097,12 +1122,7 @@ static bte_status sis_one(bte_ctx *c) {
     a.ediff_in = c->ediff[c->ecur];
     a.ediff_out = c->ediff[c->ecur ^ 1];
     cudaError_t e;
-    if (c->tiled) {
-        e = launch_step_tiled(a, c->plan, c->stream);
-        c->plan.stall = 0;
-    } else {
-        e = launch_step_generic(a, c->storage, c->limiter, c->stream);
-    }
+    e = launch_forward(c, a, c->stream);
     if (e != cudaSuccess) return fail(c, BTE_ECUDA, "forward step launch: %s", cudaGetErrorString(e));
     CU(c, launch_sis_sweep(a, static_cast<const float *>(c->e[c->cur]), static_cast<float *>(c->e[c->cur ^ 1]),
                            c->stream));
@@ -1119,12 +1139,7 @@ static bte_status sis_one(bte_ctx *c) {
     b.e_out = c->e[c->cur ^ 1];
     b.ediff_in = c->ediff[c->ecur];
     b.ediff_out = c->ediff[c->ecur ^ 1];
-    if (c->tiled) {
-        e = launch_step_tiled(b, c->plan, c->stream);
-        c->plan.stall = 0;
-    } else {
-        e = launch_step_generic(b, c->storage, c->limiter, c->stream);
-    }
+    e = launch_forward(c, b, c->stream);
     if (e != cudaSuccess) return fail(c, BTE_ECUDA, "forward step launch: %s", cudaGetErrorString(e));
     double kb = 0.0;
     for (int k = 0; k < c->nb; ++k) kb += c->C[k] * c->v[k] * c->v[k] * c->tau[k];

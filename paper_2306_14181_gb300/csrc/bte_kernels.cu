@@ -1,7 +1,7 @@
 // Generic kernels of the GB300 explicit DOM transient step (arXiv 2306.14181, Sec. 4):
 // equilibrium fill, the per-(cell, band) forward step for any grid shape, the moment-only
 // pass, the T_L finalisation and the FP64 diagnostics.  The shared-memory tiled forward
-// kernel lives in bte_tiled.cu.
+// kernel lives in bte_tiled.cu, the register-streaming one in bte_stream.cu.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -12,7 +12,9 @@
 namespace bte {
 
 // ------------------------------------------------------------------------------------------
-// Generic forward step: one thread per (cell, band), looping over the band's directions.
+// Generic forward step: one thread per (cell, band), looping over the band's directions (1-D grids and
+// 16-bit states the tiled kernel does not take, and planes too large for the streaming kernel's 32-bit
+// indices; other FP32 grids run bte_stream_kernel.cuh).
 // Eq. (disretized_transientBTE) with the limited upwind face value of Sec. 4.1, in upwind
 // orientation: with sg = sign(nu_a) and u_j = e(i + j sg),
 //   e_out = u_0 + L(u_0 - u_-1, u_1 - u_0)/2,  e_in = u_-1 + L(u_-1 - u_-2, u_0 - u_-1)/2,
