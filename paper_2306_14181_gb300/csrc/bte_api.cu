@@ -35,6 +35,7 @@ struct bte_ctx {
     int nb = 0, nd = 0;
     std::vector<double> C, v, tau, s, w;
     std::vector<int> mirror;  // [3][nd], -1 = none
+    int mom_rule = 0;         // structure of the directions for the moments: 0 any, 1 octants, 2 along x
     int bc[6] = {0, 0, 0, 0, 0, 0};
     double Tw[6] = {0, 0, 0, 0, 0, 0};
     double jump[3] = {0, 0, 0};  // temperature difference across each periodic pair (Sec. 2.2 (iv))
@@ -263,6 +264,7 @@ static bte_status build_quadrature(const bte_quadrature *q, int dim, bte_ctx *c)
     }
     c->nd = (int)c->w.size();
     (void)dim;
+    c->mom_rule = q->kind == BTE_QUAD_OCTANT ? 1 : (q->kind == BTE_QUAD_GL1D_POLAR ? 2 : 0);
     // mirror partners: direction with component a negated (same weight)
     c->mirror.assign(3 * c->nd, -1);
     for (int a = 0; a < 3; ++a)
@@ -328,9 +330,14 @@ static bte_status refresh_moments(bte_ctx *c) {
     StepArgs a = make_args(c);
     a.e_in = c->e[c->cur];
     a.ediff_out = c->ediff[c->ecur ^ 1];
-    CU(c, launch_moment_only(a, c->storage, c->stream));
     c->ecur ^= 1;
-    CU(c, launch_finalize(a, c->nb, c->TL, c->stream));
+    if (c->storage == BTE_STORE_F32 && c->dim >= 2) {
+        CU(c, launch_moment_rows(a, c->stream));
+        CU(c, launch_tl_and_walls(a, c->nb, static_cast<const float *>(a.e_in), c->TL, c->stream));
+    } else {
+        CU(c, launch_moment_only(a, c->storage, c->stream));
+        CU(c, launch_finalize(a, c->nb, c->TL, c->stream));
+    }
     c->tl_corrected = false;
     c->iface_pure = true;
     if (c->peer) TRY(iface_mix(c));
@@ -1053,7 +1060,7 @@ extern "C" bte_status bte_moments(bte_ctx *c, double *dT, double *dTL, double *q
     CU(c, cudaMemsetAsync(c->dflag, 0, sizeof(int), c->stream));
     StepArgs a = make_args(c);
     a.e_in = c->e[c->cur];
-    CU(c, launch_moments64(a, c->storage, c->d_w, c->d_s, c->d_v, c->d_invtau, c->sumC, c->D, o, c->stream));
+    CU(c, launch_moments64(a, c->storage, c->mom_rule, c->d_w, c->d_s, c->d_v, c->d_invtau, c->sumC, c->D, o, c->stream));
     int flag = 0;
     CU(c, cudaMemcpyAsync(&flag, c->dflag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     if (dT) CU(c, cudaMemcpyAsync(dT, o.T, c->ncell * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -1076,7 +1083,7 @@ extern "C" bte_status bte_energy(bte_ctx *c, double *E_total, double wall_flux[6
     a.ediff_in = c->ediff[c->ecur];
     DiagOut o2 = o;
     o2.T = o2.TL = o2.q = nullptr;
-    CU(c, launch_moments64(a, c->storage, c->d_w, c->d_s, c->d_v, c->d_invtau, c->sumC, c->D, o2, c->stream));
+    CU(c, launch_moments64(a, c->storage, c->mom_rule, c->d_w, c->d_s, c->d_v, c->d_invtau, c->sumC, c->D, o2, c->stream));
     CU(c, launch_sum64(o.cellE, c->ncell, sums, sums + 1024, c->stream));
     CU(c, launch_wallflux64(a, c->storage, c->limiter, c->d_w, c->d_s, c->d_v, o, c->stream));
     for (int wl = 0; wl < 6; ++wl)
@@ -1105,7 +1112,7 @@ static bte_status moments_on_device(bte_ctx *c, const DiagOut &o) {
     DiagOut o2 = o;
     o2.TL = nullptr;
     o2.cellE = nullptr;
-    CU(c, launch_moments64(a, c->storage, c->d_w, c->d_s, c->d_v, c->d_invtau, c->sumC, c->D, o2, c->stream));
+    CU(c, launch_moments64(a, c->storage, c->mom_rule, c->d_w, c->d_s, c->d_v, c->d_invtau, c->sumC, c->D, o2, c->stream));
     return BTE_OK;
 }
 

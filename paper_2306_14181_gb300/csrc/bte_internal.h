@@ -76,6 +76,7 @@ struct StepArgs {
 // Launchers (bte_kernels.cu).  All return the launch error (cudaGetLastError()).
 cudaError_t launch_fill(const StepArgs &a, int storage, const double *dT0, float *R_out, cudaStream_t s);
 cudaError_t launch_moment_only(const StepArgs &a, int storage, cudaStream_t s);
+cudaError_t launch_moment_rows(const StepArgs &a, cudaStream_t s);  // FP32: the partials alone, no wall values
 cudaError_t launch_step_generic(const StepArgs &a, int storage, int limiter, cudaStream_t s);
 cudaError_t launch_finalize(const StepArgs &a, int G, float *TL_out, cudaStream_t s);
 // Persistent single-CTA run of nsteps steps of a 1-D FP32 problem (bte_persist.cu): e_io in
@@ -94,7 +95,8 @@ struct DiagOut {
     double *wallpart;         // [6][nb][wc_max] partial wall flows
     int *nonfinite;           // flag
 };
-cudaError_t launch_moments64(const StepArgs &a, int storage, const double *w, const double *sv, const double *v,
+// rule: the directions' structure (kMom* in bte_kernels.cu): 0 any, 1 the octant rule, 2 along x only.
+cudaError_t launch_moments64(const StepArgs &a, int storage, int rule, const double *w, const double *sv, const double *v,
                              const double *invtau, double sumC, double D, DiagOut o, cudaStream_t s);
 cudaError_t launch_wallflux64(const StepArgs &a, int storage, int limiter, const double *w, const double *sv,
                               const double *v, DiagOut o, cudaStream_t s);

@@ -145,6 +145,51 @@ __global__ void __launch_bounds__(256) k_moment_only(const StepArgs a) {
     store_iso_codes<Cd>(a, k, i, c, rho_i, b);
 }
 
+// T_L moment partials of an FP32 state without stepping (after an equilibrium fill, a state upload or a
+// sweep): P[k][i] = sum_d w_d e/tau_k.  Bound by DRAM: a thread takes VL neighbouring cells (16 bytes)
+// of every fourth direction with eight loads in flight, and the four direction groups of a block are
+// added in order.  256^2, 40 x 128 (1.34 GB): 693 us by k_moment_only, a thread a cell and band.  (1-D
+// and 16-bit states keep that one: their T_L seeds runs that show its last bits.)
+template <int VL>
+__global__ void __launch_bounds__(256) k_moment_rows(const StepArgs a) {
+    __shared__ float part[4][VL][64];
+    const int lane = threadIdx.x & 63, grp = threadIdx.x >> 6;
+    const long long i = ((long long)blockIdx.x * 64 + lane) * VL;
+    const bool valid = i < a.ncell;
+    const int k = blockIdx.y;
+    float s[VL];
+    #pragma unroll
+    for (int j = 0; j < VL; ++j) s[j] = 0.f;
+    if (valid) {
+        const float *e = static_cast<const float *>(a.e_in) + (long long)k * a.nd * a.ncell + i;
+        const float *wm = a.wmom + (long long)k * a.nd;
+        #pragma unroll 8
+        for (int d = grp; d < a.nd; d += 4) {
+            const float wd = __ldg(wm + d);
+            if constexpr (VL == 4) {
+                const float4 f = __ldcs(reinterpret_cast<const float4 *>(e + (long long)d * a.ncell));
+                s[0] = fmaf(wd, f.x, s[0]);
+                s[1] = fmaf(wd, f.y, s[1]);
+                s[2] = fmaf(wd, f.z, s[2]);
+                s[3] = fmaf(wd, f.w, s[3]);
+            } else {
+                s[0] = fmaf(wd, __ldcs(e + (long long)d * a.ncell), s[0]);
+            }
+        }
+    }
+    #pragma unroll
+    for (int j = 0; j < VL; ++j) part[grp][j][lane] = s[j];
+    __syncthreads();
+    if (grp == 0 && valid) {
+        #pragma unroll
+        for (int j = 0; j < VL; ++j) {
+            #pragma unroll
+            for (int g = 1; g < 4; ++g) s[j] += part[g][j][lane];
+            a.P[(long long)k * a.ncell + i + j] = s[j];
+        }
+    }
+}
+
 // T_L_i = (sum_g P[g][i]) / sum_k C_k/tau_k, Eq. (BTE_get_e0), summed in fixed g order.
 __global__ void __launch_bounds__(256) k_finalize(const float *__restrict__ P, int G, long long ncell, float invD,
                                                   float *__restrict__ TL) {
@@ -214,6 +259,13 @@ cudaError_t launch_moment_only(const StepArgs &a, int storage, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+cudaError_t launch_moment_rows(const StepArgs &a, cudaStream_t s) {
+    // four cells a thread where planes are multiples of four cells (their loads are then aligned)
+    if (a.ncell % 4 == 0) k_moment_rows<4><<<dim3((unsigned)((a.ncell / 4 + 63) / 64), (unsigned)a.nb), 256, 0, s>>>(a);
+    else k_moment_rows<1><<<dim3((unsigned)((a.ncell + 63) / 64), (unsigned)a.nb), 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 // Direction groups of the generic step: one while cells x bands give at least 4096 blocks of 256
 // threads' worth of work, else more (up to 32, no more than the directions), so that small grids
 // still spread over the GPU's SMs.  In 1-D and 2-D at least 16 when there are 32 directions or
@@ -253,45 +305,165 @@ cudaError_t launch_finalize(const StepArgs &a, int G, float *TL_out, cudaStream_
 // ------------------------------------------------------------------------------------------
 
 // Per-cell moments of Eq. (getTQ) and Eq. (BTE_get_e0), FP64 accumulation.
-template <int S>
-__global__ void __launch_bounds__(256) k_moments64(const StepArgs a, const double *w, const double *sv,
-                                                   const double *v, const double *invtau, double sumC, double D,
-                                                   DiagOut o) {
+//
+// Bound by the FP64 pipe (two lanes a clock an SM), so the kernel spends as few FP64 operations a state
+// value as it can: the conversion from FP32 or 16 bits is integer arithmetic; w and w s come from a shared
+// table (one fused operation each for the sum and the three flux components); with the octant rule the
+// eight directions that differ in signs are added and subtracted first (18 additions and 4 fused
+// operations for eight values); with the 1-D polar rule only the x flux is formed, and no flux where no
+// caller asks for one.  16-bit states sum the codes; the reference's share, rho s_k sum w, is added
+// once a cell.  Each of a block's 8 warps takes a part of the (band, direction) list of 32 cells, so small
+// grids fill the GPU too; the parts are added in order.  bte_moments of the 203 x 157, 24 x 96 hot
+// spot 1260 -> 711 us, of 256^2, 40 x 128 5234 -> 2874 us (before: a thread a cell, five FP64 operations and
+// a conversion a value).
+constexpr int kMomTab = 256;  // directions (octant rule: per octant) whose weights fit the shared table
+enum { kMomGeneral = 0, kMomOctant = 1, kMomAxis = 2 };
+
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t u = __float_as_uint(f), m = u & 0x7fffffffu;
+    if (m != 0u && m < 0x00800000u) return (double)f;  // a subnormal
+    const uint32_t hi = m == 0u ? u : ((u & 0x80000000u) | ((m >> 3) + 0x38000000u));
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+// one stored value (without its reference) and whether it is an infinity or a NaN
+template <int S> struct Raw;
+template <> struct Raw<kStoreF32> {
+    static __device__ __forceinline__ float ld(const void *p, long long j, uint32_t &bad) {
+        const float f = __ldg(static_cast<const float *>(p) + j);
+        bad |= (uint32_t)((__float_as_uint(f) & 0x7f800000u) == 0x7f800000u);
+        return f;
+    }
+};
+template <> struct Raw<kStoreF16> {
+    static __device__ __forceinline__ float ld(const void *p, long long j, uint32_t &bad) {
+        const unsigned short u = __ldg(static_cast<const unsigned short *>(p) + j);
+        bad |= (uint32_t)((u & 0x7c00u) == 0x7c00u);
+        return __half2float(__ushort_as_half(u));
+    }
+};
+template <> struct Raw<kStoreBF16> {
+    static __device__ __forceinline__ float ld(const void *p, long long j, uint32_t &bad) {
+        const uint32_t u = __ldg(static_cast<const unsigned short *>(p) + j);
+        bad |= (uint32_t)((u & 0x7f80u) == 0x7f80u);
+        return __uint_as_float(u << 16);
+    }
+};
+
+// MODE: kMomOctant (directions o nq + q, o the signs), kMomAxis (only s_x differs from 0), else any
+// rule.  Q: the flux is wanted.  sum0: sum_d w, sum_d w s.
+template <int S, int MODE, bool Q>
+__global__ void __launch_bounds__(256) k_moments64(const StepArgs a, const double *__restrict__ w,
+                                                   const double *__restrict__ sv, const double *__restrict__ v,
+                                                   const double *__restrict__ invtau, double sumC, double D, DiagOut o) {
     using Cd = Codec<S>;
-    using T = typename Cd::T;
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.ncell) return;
-    const T *e = static_cast<const T *>(a.e_in);
-    const float rho_i = rho_at<Cd>(a.R, a.invTs, i);
-    double et = 0.0, tl = 0.0, qx = 0.0, qy = 0.0, qz = 0.0;
-    bool bad = false;
-    for (int k = 0; k < a.nb; ++k) {
-        const BandConst b = a.band[k];
-        double sk = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
-        for (int d = 0; d < a.nd; ++d) {
-            const double ed = Cd::ld64(e, ((long long)k * a.nd + d) * a.ncell + i, b, rho_i);
-            bad |= !isfinite(ed);
-            const double we = w[d] * ed;
-            sk += we;
-            sx += we * sv[3 * d];
-            sy += we * sv[3 * d + 1];
-            sz += we * sv[3 * d + 2];
+    constexpr int NG = 8, NQ = MODE == kMomAxis ? 1 : 3;
+    __shared__ double tab[4][kMomTab];
+    __shared__ double red[5][NG][32];
+    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    const int n = MODE == kMomOctant ? a.nd / 8 : a.nd;  // directions, or direction octets, a band
+    const bool shared = n <= kMomTab;
+    for (int d = threadIdx.x; shared && d < n; d += 256) {
+        tab[0][d] = w[d];
+        #pragma unroll
+        for (int x = 0; x < 3; ++x) tab[1 + x][d] = w[d] * sv[3 * d + x];
+    }
+    __syncthreads();
+    const long long i = (long long)blockIdx.x * 32 + lane;
+    const bool valid = i < a.ncell;
+    const long long ii = valid ? i : a.ncell - 1;
+    double et = 0.0, tl = 0.0, q[3] = {0.0, 0.0, 0.0};
+    uint32_t bad = 0;
+    auto weight = [&](int x, int d) { return shared ? tab[x][d] : (x == 0 ? w[d] : w[d] * sv[3 * d + x - 1]); };
+    const int np = a.nb * n, p1 = (int)((long long)(grp + 1) * np / NG);
+    int p = (int)((long long)grp * np / NG);
+    while (p < p1) {
+        const int k = p / n, d0 = p - k * n, d1 = min(n, d0 + p1 - p);
+        const long long base = (long long)k * a.nd * a.ncell + ii;
+        double s0 = 0.0, s[3] = {0.0, 0.0, 0.0};
+        if constexpr (MODE == kMomOctant) {
+            #pragma unroll 2
+            for (int d = d0; d < d1; ++d) {
+                double e[8];
+                #pragma unroll
+                for (int oc = 0; oc < 8; ++oc) e[oc] = widen(Raw<S>::ld(a.e_in, base + (long long)(oc * n + d) * a.ncell, bad));
+                double u[4], x = 0.0;
+                #pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    u[j] = e[2 * j] + e[2 * j + 1];
+                    if constexpr (Q) x += e[2 * j] - e[2 * j + 1];
+                }
+                const double z0 = u[0] + u[1], z1 = u[2] + u[3];
+                s0 = fma(weight(0, d), z0 + z1, s0);
+                if constexpr (Q) {
+                    s[0] = fma(weight(1, d), x, s[0]);
+                    s[1] = fma(weight(2, d), (u[0] - u[1]) + (u[2] - u[3]), s[1]);
+                    s[2] = fma(weight(3, d), z0 - z1, s[2]);
+                }
+            }
+        } else {
+            #pragma unroll 8
+            for (int d = d0; d < d1; ++d) {
+                const double e = widen(Raw<S>::ld(a.e_in, base + (long long)d * a.ncell, bad));
+                s0 = fma(weight(0, d), e, s0);
+                if constexpr (Q) {
+                    #pragma unroll
+                    for (int x = 0; x < NQ; ++x) s[x] = fma(weight(1 + x, d), e, s[x]);
+                }
+            }
         }
-        et += sk;
-        tl += invtau[k] * sk;
-        qx += v[k] * sx;
-        qy += v[k] * sy;
-        qz += v[k] * sz;
+        const double sc = Cd::kRef ? (double)a.band[k].scale : 1.0;
+        et = fma(sc, s0, et);
+        tl = fma(sc * invtau[k], s0, tl);
+        if constexpr (Q) {
+            #pragma unroll
+            for (int x = 0; x < NQ; ++x) q[x] = fma(sc * v[k], s[x], q[x]);
+        }
+        p += d1 - d0;
     }
-    if (bad) atomicOr(o.nonfinite, 1);
-    if (o.T) o.T[i] = et / sumC;
-    if (o.TL) o.TL[i] = tl / D;
-    if (o.q) {
-        o.q[i] = qx;
-        o.q[a.ncell + i] = qy;
-        o.q[2 * a.ncell + i] = qz;
+    if constexpr (Cd::kRef) {
+        // the references' share, by group 0: rho sum_k s_k (1, 1/tau_k, v_k) times sum_d w (1, 1, s)
+        const float rho = rho_at<Cd>(a.R, a.invTs, ii);
+        bad |= (uint32_t)!isfinite(rho);
+        if (grp == 0) {
+            double w0 = 0.0, ws[3] = {0.0, 0.0, 0.0}, k0 = 0.0, kt = 0.0, kv = 0.0;
+            for (int d = 0; d < a.nd; ++d) {
+                w0 += w[d];
+                #pragma unroll
+                for (int x = 0; x < 3; ++x) ws[x] = fma(w[d], sv[3 * d + x], ws[x]);
+            }
+            for (int k = 0; k < a.nb; ++k) {
+                const double sc = (double)a.band[k].scale;
+                k0 += sc;
+                kt = fma(sc, invtau[k], kt);
+                kv = fma(sc, v[k], kv);
+            }
+            et = fma((double)rho * w0, k0, et);
+            tl = fma((double)rho * w0, kt, tl);
+            if constexpr (Q) {
+                #pragma unroll
+                for (int x = 0; x < NQ; ++x) q[x] = fma((double)rho * ws[x], kv, q[x]);
+            }
+        }
     }
-    if (o.cellE) o.cellE[i] = et;
+    red[0][grp][lane] = et;
+    red[1][grp][lane] = tl;
+    #pragma unroll
+    for (int x = 0; x < 3; ++x) red[2 + x][grp][lane] = q[x];
+    if (bad && valid) atomicOr(o.nonfinite, 1);
+    __syncthreads();
+    // outputs: warp r adds the parts of quantity r in order
+    if (grp < 5 && valid) {
+        double t = 0.0;
+        for (int g = 0; g < NG; ++g) t += red[grp][g][lane];
+        if (grp == 0) {
+            if (o.T) o.T[i] = t / sumC;
+            if (o.cellE) o.cellE[i] = t;
+        } else if (grp == 1) {
+            if (o.TL) o.TL[i] = t / D;
+        } else if (o.q) {
+            o.q[(long long)(grp - 2) * a.ncell + i] = t;
+        }
+    }
 }
 
 template <class Cd>
@@ -369,12 +541,24 @@ __global__ void __launch_bounds__(256) k_wallflux64(const StepArgs a, int wall, 
     o.wallpart[((long long)wall * a.nb + k) * a.wc_max + j] = F;
 }
 
-cudaError_t launch_moments64(const StepArgs &a, int storage, const double *w, const double *sv, const double *v,
+template <int S>
+static void moments64_s(const StepArgs &a, int rule, const double *w, const double *sv, const double *v,
+                        const double *invtau, double sumC, double D, const DiagOut &o, cudaStream_t s) {
+    const unsigned g = (unsigned)((a.ncell + 31) / 32);
+#define BTE_MOM(M_) \
+    (o.q ? k_moments64<S, M_, true><<<g, 256, 0, s>>>(a, w, sv, v, invtau, sumC, D, o) \
+         : k_moments64<S, M_, false><<<g, 256, 0, s>>>(a, w, sv, v, invtau, sumC, D, o))
+    if (rule == kMomOctant) BTE_MOM(kMomOctant);
+    else if (rule == kMomAxis) BTE_MOM(kMomAxis);
+    else BTE_MOM(kMomGeneral);
+#undef BTE_MOM
+}
+
+cudaError_t launch_moments64(const StepArgs &a, int storage, int rule, const double *w, const double *sv, const double *v,
                              const double *invtau, double sumC, double D, DiagOut o, cudaStream_t s) {
-    const dim3 g = cell_grid(a.ncell, 1);
-    if (storage == kStoreF32) k_moments64<kStoreF32><<<g, 256, 0, s>>>(a, w, sv, v, invtau, sumC, D, o);
-    else if (storage == kStoreF16) k_moments64<kStoreF16><<<g, 256, 0, s>>>(a, w, sv, v, invtau, sumC, D, o);
-    else k_moments64<kStoreBF16><<<g, 256, 0, s>>>(a, w, sv, v, invtau, sumC, D, o);
+    if (storage == kStoreF32) moments64_s<kStoreF32>(a, rule, w, sv, v, invtau, sumC, D, o, s);
+    else if (storage == kStoreF16) moments64_s<kStoreF16>(a, rule, w, sv, v, invtau, sumC, D, o, s);
+    else moments64_s<kStoreBF16>(a, rule, w, sv, v, invtau, sumC, D, o, s);
     return cudaGetLastError();
 }
 

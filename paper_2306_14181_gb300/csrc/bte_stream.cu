@@ -13,7 +13,7 @@ namespace stream {
 // Finalize pass of a step: a block is 64 items by 4 groups; group g takes rows (or directions) g,
 // g + 4, ... and group 0 adds the four sums in order, so the result is fixed for a given plan.
 // The first tblocks blocks form T_L_i = (sum of the moment partials of cell i) / sum_k C_k/tau_k.
-// The others form the diffuse-wall values of e^{n+1}, Eq. (diff_bound), from the stored state: sum over
+// The others form the diffuse-wall values, Eq. (diff_bound), from the stored state: sum over
 // the leaving directions of w |s.n| e / sum_in w|s.n|.
 constexpr int kItems = 64, kGroups = 4;
 
@@ -24,7 +24,7 @@ struct WallList {
 };
 
 __global__ void __launch_bounds__(kItems * kGroups) k_finalize_stream(const StepArgs a, int rows, int tblocks,
-                                                                      const WallList wl, float *TL_out) {
+                                                                      const WallList wl, const float *state, float *TL_out) {
     __shared__ float part[kGroups][kItems];
     const int lane = threadIdx.x % kItems, grp = threadIdx.x / kItems;
     if ((int)blockIdx.x < tblocks) {
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kItems * kGroups) k_finalize_stream(const Step
         const int y = ax == 0 ? ja : (ax == 1 ? (side ? a.n[1] - 1 : 0) : jb);
         const int z = ax == 2 ? (side ? a.n[2] - 1 : 0) : jb;
         const long long i = ((long long)z * a.n[1] + y) * a.n[0] + x;
-        const float *e = static_cast<const float *>(a.e_out) + (long long)k * a.nd * a.ncell + i;
+        const float *e = state + (long long)k * a.nd * a.ncell + i;
         const float *wd = a.wdiff + wall * a.nd;
         #pragma unroll 4
         for (int d = grp; d < a.nd; d += kGroups) {
@@ -197,7 +197,7 @@ cudaError_t launch_step_stream(const StepArgs &a, const StreamPlan &plan, cudaSt
     return cudaGetLastError();
 }
 
-cudaError_t launch_finalize_stream(const StepArgs &a, const StreamPlan &plan, float *TL_out, cudaStream_t s) {
+cudaError_t launch_tl_and_walls(const StepArgs &a, int rows, const float *state, float *TL_out, cudaStream_t s) {
     WallList wl;
     wl.n = 0;
     wl.first[0] = 0;
@@ -210,8 +210,12 @@ cudaError_t launch_finalize_stream(const StepArgs &a, const StreamPlan &plan, fl
     }
     const int tblocks = (int)((a.ncell + kItems - 1) / kItems);
     const unsigned blocks = (unsigned)tblocks + (unsigned)(wl.first[wl.n] / kItems) * (unsigned)a.nb;
-    k_finalize_stream<<<blocks, kItems * kGroups, 0, s>>>(a, a.nb * plan.nchunk, tblocks, wl, TL_out);
+    k_finalize_stream<<<blocks, kItems * kGroups, 0, s>>>(a, rows, tblocks, wl, state, TL_out);
     return cudaGetLastError();
+}
+
+cudaError_t launch_finalize_stream(const StepArgs &a, const StreamPlan &plan, float *TL_out, cudaStream_t s) {
+    return launch_tl_and_walls(a, a.nb * plan.nchunk, static_cast<const float *>(a.e_out), TL_out, s);
 }
 
 }  // namespace bte
