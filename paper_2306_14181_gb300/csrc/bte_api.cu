@@ -954,6 +954,7 @@ static cudaError_t launch_forward(bte_ctx *c, const StepArgs &a, cudaStream_t st
         return e;
     }
     if (c->streamed) return launch_step_stream(a, c->splan, strm);
+    if (c->dim == 1) return launch_step_1d(a, c->storage, c->limiter, strm);
     return launch_step_generic(a, c->storage, c->limiter, strm);
 }
 
@@ -981,6 +982,7 @@ static bte_status step_one(bte_ctx *c, cudaStream_t strm) {
         float *TL_next = c->R;
         if (c->tiled) e = launch_finalize_tiled(a, c->plan, c->storage, TL_next, strm);
         else if (c->streamed) e = launch_finalize_stream(a, c->splan, TL_next, strm);
+        else if (c->dim == 1) e = launch_finalize_1d(a, c->storage, TL_next, strm);
         else e = launch_finalize(a, c->G, TL_next, strm);
         if (e != cudaSuccess) return fail(c, BTE_ECUDA, "finalize launch: %s", cudaGetErrorString(e));
         if (c->prof) TRY(prof_event(c, &ev));

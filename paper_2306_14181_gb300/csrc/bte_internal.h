@@ -78,6 +78,9 @@ cudaError_t launch_fill(const StepArgs &a, int storage, const double *dT0, float
 cudaError_t launch_moment_only(const StepArgs &a, int storage, cudaStream_t s);
 cudaError_t launch_moment_rows(const StepArgs &a, cudaStream_t s);  // FP32: the partials alone, no wall values
 cudaError_t launch_step_generic(const StepArgs &a, int storage, int limiter, cudaStream_t s);
+// The 1-D step of any storage: the update, then T_L and the diffuse-wall values from e_out.
+cudaError_t launch_step_1d(const StepArgs &a, int storage, int limiter, cudaStream_t s);
+cudaError_t launch_finalize_1d(const StepArgs &a, int storage, float *TL_out, cudaStream_t s);
 cudaError_t launch_finalize(const StepArgs &a, int G, float *TL_out, cudaStream_t s);
 // Persistent single-CTA run of nsteps steps of a 1-D FP32 problem (bte_persist.cu): e_io in
 // place, T_L and the diffuse-wall values of the final state out; amps[s] the source amplitude
