@@ -32,8 +32,25 @@ namespace bte {
 namespace tiled {
 
 // ---- finalize passes ---------------------------------------------------------------------
-// T_L_i = (sum over the segments of i's tile, in order) / sum_k C_k / tau_k
-__global__ void __launch_bounds__(256) k_finalize_tiled(const StepArgs a, const TiledArgs p, float *TL) {
+// One launch: blocks 0 .. tblocks-1 form T_L_i = (sum over the segments of i's tile, in order) /
+// sum_k C_k / tau_k, the others the wall ghost values of e^{n+1}.  Both are short chains of dependent
+// loads, so they run side by side (256^2, 40 x 128, three diffuse walls: 24 -> 14 us).
+struct WallList {
+    int w[6];
+    int blocks;  // of 256 cells, a wall and band
+};
+
+template <int S>
+__device__ __forceinline__ void wall_values(const StepArgs &a, const TiledArgs &p, int wall, int k, long long j);
+
+template <int S>
+__global__ void __launch_bounds__(256) k_finalize_tiled(const StepArgs a, const TiledArgs p, float *TL, int tblocks,
+                                                        const WallList wls) {
+    if ((int)blockIdx.x >= tblocks) {
+        const int q = blockIdx.x - tblocks, wk = q / wls.blocks, w = wk / a.nb;
+        wall_values<S>(a, p, wls.w[w], wk - w * a.nb, (long long)(q - wk * wls.blocks) * 256 + threadIdx.x);
+        return;
+    }
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.ncell) return;
     const int nx = a.n[0], ny = a.n[1];
@@ -46,8 +63,8 @@ __global__ void __launch_bounds__(256) k_finalize_tiled(const StepArgs a, const 
     const int g0 = p.tile_seg0[tile], g1 = p.tile_seg0[tile + 1];
     const float *P = a.P + li;
     float s = 0.f;
-    #pragma unroll 8
-    for (int g = g0; g < g1; ++g) s += P[(size_t)g * p.tcells];
+    #pragma unroll 16
+    for (int g = g0; g < g1; ++g) s += __ldcs(P + (size_t)g * p.tcells);
     TL[i] = s * a.invD;
 }
 
@@ -55,20 +72,13 @@ __global__ void __launch_bounds__(256) k_finalize_tiled(const StepArgs a, const 
 // (sum over the band-k segments of the cell's tile) / sum_in w|s.n|.  With 16-bit storage the
 // value is coded against the wall cell's new reference rho = T_L^n / T_scale, and thermalizing
 // y/z walls get their emission C_k T_w / W coded the same way.
-struct WallList {
-    int w[6];
-};
-
 template <int S>
-__global__ void __launch_bounds__(256) k_ediff_tiled(const StepArgs a, const TiledArgs p, const WallList wls) {
+__device__ __forceinline__ void wall_values(const StepArgs &a, const TiledArgs &p, int wall, int k, long long j) {
     using T = typename St<S>::T;
-    const int wall = wls.w[blockIdx.z];
     const int ax = wall >> 1, side = wall & 1;
     const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
     const int n0 = ax == 0 ? ny : nx;            // fastest wall-cell coordinate extent
     const int n1 = ax == 2 ? ny : nz;
-    const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = blockIdx.y;
     if (j >= (long long)n0 * n1) return;
     const int ja = (int)(j % n0), jb = (int)(j / n0);
     int x, y, z;
@@ -85,12 +95,12 @@ __global__ void __launch_bounds__(256) k_ediff_tiled(const StepArgs a, const Til
         const int yl = y - ty * p.ty, zl = z - tz * p.tz;
         const int slot = ax == 0 ? zl * p.ty + yl : (ax == 1 ? zl * p.nxt + x : yl * p.nxt + x);
         float s = 0.f;
-        for (int jj = 0; jj < p.J; ++jj) {
-            const int u = jj * p.ntiles + tile;
-            const int p0 = part_begin(p, jj), p1 = part_begin(p, jj + 1);
-            if (p0 >= p1) continue;
-            const int b0 = p0 / a.nd, b1 = (p1 - 1) / a.nd;
-            if (k < b0 || k > b1) continue;
+        // the parts that hold planes of band k, in order: part_begin(j) is the floor of j np / J
+        int jj = (int)((long long)k * a.nd * p.J / p.np);
+        for (int p0 = part_begin(p, jj), p1; jj < p.J && p0 < (k + 1) * a.nd; ++jj, p0 = p1) {
+            p1 = part_begin(p, jj + 1);
+            if (p0 >= p1 || p1 <= k * a.nd) continue;
+            const int u = jj * p.ntiles + tile, b0 = p0 / a.nd;
             s += p.PW[((size_t)(p.unit_seg0[u] + k - b0) * p.nwd + p.wslot[wall]) * p.tw + slot];
         }
         v = s * a.inv_den[wall];
@@ -134,10 +144,10 @@ __global__ void k_fill_isorows(const StepArgs a, int nx, float *rows) {
 }
 
 // ---- dispatch -------------------------------------------------------------------------------
-StepKernel pick(int storage, int lim, int nx, int dim, bool sr) {
-    if (storage == kStoreF32) return dim == 2 ? pick_f32_2d(lim, nx) : pick_f32_3d(lim, nx);
-    if (storage == kStoreF16) return dim == 2 ? pick_f16_2d(lim, nx, sr) : pick_f16_3d(lim, nx, sr);
-    return dim == 2 ? pick_bf16_2d(lim, nx, sr) : pick_bf16_3d(lim, nx, sr);
+StepKernel pick(int storage, int lim, Rows r, int dim, bool sr) {
+    if (storage == kStoreF32) return dim == 2 ? pick_f32_2d(lim, r) : pick_f32_3d(lim, r);
+    if (storage == kStoreF16) return dim == 2 ? pick_f16_2d(lim, r, sr) : pick_f16_3d(lim, r, sr);
+    return dim == 2 ? pick_bf16_2d(lim, r, sr) : pick_bf16_3d(lim, r, sr);
 }
 
 template <class V>
@@ -206,9 +216,6 @@ bool tiled_plan(int dim, const int n[3], int nb, int nd, int storage, int limite
         const int c = std::atoi(env);
         if (c >= 1 && c <= 1024) plan.chunk = c;
     }
-    // rows shorter than the capacity lie at another stride in global memory than in the box:
-    // one bulk copy a row
-    if (gxn != nx) plan.chunk = 1;
     plan.ty = TY;
     plan.tz = TZ;
     plan.threads = (ncw + kProducerWarps) * 32;
@@ -219,7 +226,7 @@ bool tiled_plan(int dim, const int n[3], int nb, int nd, int storage, int limite
     plan.tw = std::max(std::max(TY * TZ, nx * TZ), dim == 3 ? nx * TY : 0);
     const size_t box = (size_t)(TY + 3) * (dim == 3 ? TZ + 3 : 1) * nx * esz;
     const int V = 16 / esz;  // elements in 16 bytes
-    const size_t side_bytes = ((size_t)2 * TZ * TY * V + (size_t)2 * TZ * (TY + V)) * esz;
+    const size_t side_bytes = (size_t)2 * TZ * (TY + V + 2 * TY) * esz;
     plan.side_off = (int)((box + 127) / 128 * 128);
     plan.hdr_off = plan.side_off + (int)((side_bytes + 15) / 16 * 16);
     plan.stage_bytes = (int)((plan.hdr_off + kHdrFloats * sizeof(float) + 127) / 128 * 128);
@@ -249,7 +256,7 @@ bool tiled_plan(int dim, const int n[3], int nb, int nd, int storage, int limite
     plan.acc_off = plan.bt_off + (int)((bt_bytes + 127) / 128 * 128);
     plan.rho_off = plan.acc_off + (int)((acc_bytes + 127) / 128 * 128);
     plan.smem = plan.rho_off + (int)rho_bytes;
-    plan.kernel = (void *)pick(storage, limiter, nx, dim, sr && storage != kStoreF32);
+    plan.kernel = (void *)pick(storage, limiter, Rows{nx, gxn == nx}, dim, sr && storage != kStoreF32);
     if (!plan.kernel) {
         why = "no kernel instance";
         return false;
@@ -416,9 +423,6 @@ static bool tiled_wall_pass(const TiledPlan &plan, const int bc[6], int w) {
 cudaError_t launch_finalize_tiled(const StepArgs &a, const TiledPlan &plan, int storage, float *TL_out,
                                   cudaStream_t s) {
     const TiledArgs t = tiled_device_args(plan);
-    const unsigned nblk = (unsigned)((a.ncell + 255) / 256);
-    k_finalize_tiled<<<nblk, 256, 0, s>>>(a, t, TL_out);
-    // every wall that needs ghost values in one launch (z: the wall), x covering its cells
     WallList wl;
     int nw = 0;
     long long nwc = 0;
@@ -430,19 +434,13 @@ cudaError_t launch_finalize_tiled(const StepArgs &a, const TiledPlan &plan, int 
         nwc = std::max(nwc, m);
         wl.w[nw++] = w;
     }
-    if (nw > 0) {
-        const dim3 g((unsigned)((nwc + 255) / 256), (unsigned)a.nb, (unsigned)nw);
-        if (storage == kStoreF32) k_ediff_tiled<kStoreF32><<<g, 256, 0, s>>>(a, t, wl);
-        else if (storage == kStoreF16) k_ediff_tiled<kStoreF16><<<g, 256, 0, s>>>(a, t, wl);
-        else k_ediff_tiled<kStoreBF16><<<g, 256, 0, s>>>(a, t, wl);
-    }
+    const unsigned tblocks = (unsigned)((a.ncell + 255) / 256);
+    wl.blocks = (int)((nwc + 255) / 256);
+    const unsigned g = tblocks + (unsigned)nw * a.nb * wl.blocks;
+    if (storage == kStoreF32) k_finalize_tiled<kStoreF32><<<g, 256, 0, s>>>(a, t, TL_out, (int)tblocks, wl);
+    else if (storage == kStoreF16) k_finalize_tiled<kStoreF16><<<g, 256, 0, s>>>(a, t, TL_out, (int)tblocks, wl);
+    else k_finalize_tiled<kStoreBF16><<<g, 256, 0, s>>>(a, t, TL_out, (int)tblocks, wl);
     return cudaGetLastError();
-}
-
-int tiled_finalize_launches(const TiledPlan &plan, const int bc[6]) {
-    for (int w = 0; w < 2 * plan.dim; ++w)
-        if (tiled_wall_pass(plan, bc, w)) return 2;
-    return 1;
 }
 
 }  // namespace bte

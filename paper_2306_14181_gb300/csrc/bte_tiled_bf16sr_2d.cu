@@ -3,6 +3,6 @@
 
 namespace bte {
 namespace tiled {
-StepKernel pick_bf16sr_2d(int lim, int nx) { return pick_instance<kStoreBF16, 2, true>(lim, nx); }
+StepKernel pick_bf16sr_2d(int lim, Rows r) { return pick_instance<kStoreBF16, 2, true>(lim, r); }
 }  // namespace tiled
 }  // namespace bte

@@ -3,8 +3,8 @@
 
 namespace bte {
 namespace tiled {
-StepKernel pick_f16_2d(int lim, int nx, bool sr) {
-    return sr ? pick_f16sr_2d(lim, nx) : pick_instance<kStoreF16, 2, false>(lim, nx);
+StepKernel pick_f16_2d(int lim, Rows r, bool sr) {
+    return sr ? pick_f16sr_2d(lim, r) : pick_instance<kStoreF16, 2, false>(lim, r);
 }
 }  // namespace tiled
 }  // namespace bte

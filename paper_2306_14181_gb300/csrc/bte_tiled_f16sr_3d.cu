@@ -3,6 +3,6 @@
 
 namespace bte {
 namespace tiled {
-StepKernel pick_f16sr_3d(int lim, int nx) { return pick_instance<kStoreF16, 3, true>(lim, nx); }
+StepKernel pick_f16sr_3d(int lim, Rows r) { return pick_instance<kStoreF16, 3, true>(lim, r); }
 }  // namespace tiled
 }  // namespace bte

@@ -3,6 +3,6 @@
 
 namespace bte {
 namespace tiled {
-StepKernel pick_f32_2d(int lim, int nx) { return pick_instance<kStoreF32, 2, false>(lim, nx); }
+StepKernel pick_f32_2d(int lim, Rows r) { return pick_instance<kStoreF32, 2, false>(lim, r); }
 }  // namespace tiled
 }  // namespace bte

@@ -3,6 +3,6 @@
 
 namespace bte {
 namespace tiled {
-StepKernel pick_f32_3d(int lim, int nx) { return pick_instance<kStoreF32, 3, false>(lim, nx); }
+StepKernel pick_f32_3d(int lim, Rows r) { return pick_instance<kStoreF32, 3, false>(lim, r); }
 }  // namespace tiled
 }  // namespace bte

@@ -5,6 +5,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "bte_tiled.h"
 
 namespace bte {
@@ -81,6 +83,18 @@ template <> struct St<kStoreF16> {
     static __device__ __forceinline__ float dec(T h, float rho) { return __half2float(h) + rho; }
     static __device__ __forceinline__ float val(C c) { return __half2float(__ushort_as_half((unsigned short)c)); }
     static __device__ __forceinline__ C bits(T h) { return __half_as_ushort(h); }
+    // two codes of a 32-bit word, low half first
+    static __device__ __forceinline__ float2 val2(uint32_t u) {
+        __half2 h;
+        memcpy(&h, &u, 4);
+        return __half22float2(h);
+    }
+    static __device__ __forceinline__ uint32_t enc2(float2 v) {
+        const __half2 h = __float22half2_rn(v);
+        uint32_t u;
+        memcpy(&u, &h, 4);
+        return u;
+    }
     static __device__ __forceinline__ C enc(float v) { return __half_as_ushort(__float2half_rn(v)); }
     // stochastic rounding: 13 random bits below binary16's 10 fraction bits, then truncation
     // (exact for normal binary16 values; round to nearest in the subnormal range)
@@ -95,6 +109,15 @@ template <> struct St<kStoreBF16> {
     static __device__ __forceinline__ float dec(T h, float rho) { return __bfloat162float(h) + rho; }
     static __device__ __forceinline__ float val(C c) { return __uint_as_float(c << 16); }
     static __device__ __forceinline__ C bits(T h) { return __bfloat16_as_ushort(h); }
+    static __device__ __forceinline__ float2 val2(uint32_t u) {
+        return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+    }
+    static __device__ __forceinline__ uint32_t enc2(float2 v) {
+        const __nv_bfloat162 h = __float22bfloat162_rn(v);
+        uint32_t u;
+        memcpy(&u, &h, 4);
+        return u;
+    }
     static __device__ __forceinline__ C enc(float v) { return __bfloat16_as_ushort(__float2bfloat16_rn(v)); }
     // stochastic rounding: 16 random bits below bfloat16's 7 fraction bits, then truncation
     static __device__ __forceinline__ C enc_sr(float v, uint32_t bits) { return (__float_as_uint(v) + (bits >> 16)) >> 16; }
@@ -237,16 +260,24 @@ __device__ __forceinline__ void ld_row(float (&v)[VL], const typename St<S>::T *
         if constexpr (VL == 4) {
             const float4 f = *reinterpret_cast<const float4 *>(p);
             v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+        } else if constexpr (VL == 2) {
+            const float2 f = *reinterpret_cast<const float2 *>(p);
+            v[0] = f.x; v[1] = f.y;
         } else {
             #pragma unroll
             for (int j = 0; j < VL; ++j) v[j] = p[j];
         }
     } else {
         float f[VL], rr[VL];
-        if constexpr (VL == 4) {
+        if constexpr (VL == 2) {
+            const float2 h = Q::val2(*reinterpret_cast<const uint32_t *>(p)), g = *reinterpret_cast<const float2 *>(r);
+            f[0] = h.x; f[1] = h.y;
+            rr[0] = g.x; rr[1] = g.y;
+        } else if constexpr (VL == 4) {
             const uint2 q = *reinterpret_cast<const uint2 *>(p);
-            f[0] = Q::val(q.x & 0xffffu); f[1] = Q::val(q.x >> 16);
-            f[2] = Q::val(q.y & 0xffffu); f[3] = Q::val(q.y >> 16);
+            const float2 lo = Q::val2(q.x), hi = Q::val2(q.y);
+            f[0] = lo.x; f[1] = lo.y;
+            f[2] = hi.x; f[3] = hi.y;
             const float4 g = *reinterpret_cast<const float4 *>(r);
             rr[0] = g.x; rr[1] = g.y; rr[2] = g.z; rr[3] = g.w;
         } else {
@@ -267,22 +298,26 @@ __device__ __forceinline__ void ld_row(float (&v)[VL], const typename St<S>::T *
     }
 }
 
+// VL codes to memory: h holds them as words of two codes each (an odd last one in the low half) for 16-bit
+// storage, one value each for FP32.
+template <int S, int VL> constexpr int code_words() { return St<S>::kRef ? (VL + 1) / 2 : VL; }
 template <int S, int VL>
-__device__ __forceinline__ void st_row(typename St<S>::T *p, const typename St<S>::C (&c)[VL]) {
+__device__ __forceinline__ void st_row(typename St<S>::T *p, const typename St<S>::C (&c)[code_words<S, VL>()]) {
     using Q = St<S>;
     if constexpr (!Q::kRef) {
         if constexpr (VL == 4) *reinterpret_cast<float4 *>(p) = make_float4(c[0], c[1], c[2], c[3]);
+        else if constexpr (VL == 2) *reinterpret_cast<float2 *>(p) = make_float2(c[0], c[1]);
         else {
             #pragma unroll
             for (int j = 0; j < VL; ++j) p[j] = c[j];
         }
     } else {
-        if constexpr (VL == 4) {
-            *reinterpret_cast<uint2 *>(p) = make_uint2(c[0] | (c[1] << 16), c[2] | (c[3] << 16));
-        } else {
+        if constexpr (VL == 4) *reinterpret_cast<uint2 *>(p) = make_uint2(c[0], c[1]);
+        else if constexpr (VL == 2) *reinterpret_cast<uint32_t *>(p) = c[0];
+        else {
             unsigned short *ps = reinterpret_cast<unsigned short *>(p);
             #pragma unroll
-            for (int j = 0; j < VL; ++j) ps[j] = (unsigned short)c[j];
+            for (int j = 0; j < VL; ++j) ps[j] = (unsigned short)(c[j / 2] >> (16 * (j & 1)));
         }
     }
 }
@@ -382,21 +417,24 @@ __device__ __forceinline__ const typename St<S>::T *ghost_row_src(const StepArgs
     return static_cast<const T *>(a.ediff_in) + ((long long)wall * a.nb + q.k) * a.wc_max + (long long)other * gx;
 }
 
-// Shared-memory side arrays of a stage for the x-wall ghosts (storage format, bulk-copied):
-//   spec[wall][TZ][TY][V]   16 bytes of the mirrored direction's row at the wall (specular)
-//   dcol[wall][TZ][TY + V]  the diffuse-wall values of the tile's rows (from a 16-byte aligned start)
-// with V = 16 / sizeof(T) elements.
+// Shared-memory side arrays of a stage for the x-wall ghosts (storage format):
+//   dcol[wall][TZ][TY + V]  the diffuse-wall values of the tile's rows (bulk-copied from a 16-byte aligned
+//                           start)
+//   spec[wall][TZ][TY][2]   the mirrored direction's two cells next to a specular wall, lower x first, put
+//                           there by the lane that uses them (which loads them while it waits for the stage)
+// with V = 16 / sizeof(T) elements.  (As 16-byte bulk copies, one a row and side, the specular ghosts cost the
+// producer about 30 ns each: 128^2, 20 x 64, specular x walls, FP32 / FP16 403 / 418 us, now 191 / 223 us; 96^2 x
+// 64, FP16, 5 bands 3.44 -> 2.28 ms.)
 template <int S, int WPR, int DIM> struct Side {
     using T = typename St<S>::T;
     static constexpr int V = 16 / (int)sizeof(T);
     static constexpr int TY = Geo<DIM, WPR>::TY, TZ = Geo<DIM, WPR>::TZ, TYP = TY + V;
-    static constexpr int spec_elems = 2 * TZ * TY * V;
-    static constexpr int bytes = (spec_elems + 2 * TZ * TYP) * (int)sizeof(T);
-    static __device__ __forceinline__ T *spec(char *side, int sd, int zl, int yl) {
-        return reinterpret_cast<T *>(side) + ((sd * TZ + zl) * TY + yl) * V;
-    }
+    static constexpr int dcol_elems = 2 * TZ * TYP;
     static __device__ __forceinline__ T *dcol(char *side, int sd, int zl) {
-        return reinterpret_cast<T *>(side) + spec_elems + (sd * TZ + zl) * TYP;
+        return reinterpret_cast<T *>(side) + (sd * TZ + zl) * TYP;
+    }
+    static __device__ __forceinline__ T *spec(char *side, int sd, int zl, int yl) {
+        return reinterpret_cast<T *>(side) + dcol_elems + ((sd * TZ + zl) * TY + yl) * 2;
     }
 };
 
@@ -406,15 +444,16 @@ __device__ __forceinline__ long long dcol_src(const StepArgs &a, int sd, int k, 
     return ((long long)sd * a.nb + k) * a.wc_max + (long long)z * a.n[1] + y0;
 }
 
-template <int S, int VL, int WPR, int DIM>
+template <int S, int VL, int WPR, int DIM, bool FR>
 __device__ void producer(const StepArgs &a, const TiledArgs &p, char *smem, uint64_t *full, uint64_t *empty) {
     using T = typename St<S>::T;
     using SD = Side<S, WPR, DIM>;
     constexpr int NX = 32 * VL * WPR, TY = Geo<DIM, WPR>::TY;
     constexpr int V = SD::V;
     const int lane = threadIdx.x & 31;
-    const int gx = a.n[0], ny = a.n[1], nz = a.n[2];
-    // a row of the grid is gx <= NX cells (a multiple of 16 bytes); box rows keep the stride NX
+    const int gx = FR ? NX : a.n[0], ny = a.n[1], nz = a.n[2];
+    // a row of the grid is gx <= NX cells (a multiple of 16 bytes); box rows have the stride gx too, so
+    // runs of rows move in one copy
     const uint32_t rowb = (uint32_t)gx * sizeof(T);
     const T *e = static_cast<const T *>(a.e_in);
     const T *ed = static_cast<const T *>(a.ediff_in);
@@ -444,8 +483,6 @@ __device__ void producer(const StepArgs &a, const TiledArgs &p, char *smem, uint
         char *stage = smem + p.stage0 + (size_t)s * p.stage_bytes;
         char *side = stage + p.side_off;
         const long long pbase = (long long)q.plane * a.ncell;
-        const int ncore = q.nyt * q.nzt;
-        const bool spec[2] = {bx[0] == kBcSpecular, bx[1] == kBcSpecular};
         const bool dif[2] = {bx[0] == kBcDiffuse && nux > 0.f, bx[1] == kBcDiffuse && nux < 0.f};
         // Every box row the stencil reads is filled by exactly one bulk copy, so the byte count is
         // closed-form: core slices need all nry rows, the z-halo slices the nyt core rows.  x-wall
@@ -453,8 +490,7 @@ __device__ void producer(const StepArgs &a, const TiledArgs &p, char *smem, uint
         const int nneed = DIM == 3 ? q.nzt * nry + (nrz - q.nzt) * q.nyt : nry;
         const int ndcol = (q.nyt + V - 1) / V + 1;  // 16-byte units of a diffuse column copy
         if (lane == 0) {
-            const uint32_t bytes = (uint32_t)nneed * rowb + (spec[0] + spec[1]) * (uint32_t)ncore * 16u +
-                                   (dif[0] + dif[1]) * (uint32_t)q.nzt * ndcol * 16u + 64u;
+            const uint32_t bytes = (uint32_t)nneed * rowb + (dif[0] + dif[1]) * (uint32_t)q.nzt * ndcol * 16u + 64u;
             mbar_expect_tx(&full[s], bytes);
             // per-plane constants (64 bytes, prepared once on the device)
             bulk_g2s(stage + p.hdr_off, p.hdr + (size_t)q.plane * kHdrFloats, 64, &full[s]);
@@ -468,11 +504,11 @@ __device__ void producer(const StepArgs &a, const TiledArgs &p, char *smem, uint
         for (int w = lane; w < nrz * per; w += 32) {
             const int rz = w / per, it = w - rz * per;
             const int z = zbox0 + rz;
-            T *slice = reinterpret_cast<T *>(stage) + (size_t)rz * (TY + 3) * NX;
+            T *slice = reinterpret_cast<T *>(stage) + (size_t)rz * (TY + 3) * gx;
             if (DIM == 3 && (z < 0 || z >= nz)) {
                 if (it < q.nyt) {
                     const int y = q.y0 + it;
-                    bulk_g2s(slice + (size_t)(y - ybox0) * NX, ghost_row_src<S, NX>(a, p, q, 2, z, y, nuz), rowb, &full[s]);
+                    bulk_g2s(slice + (size_t)(y - ybox0) * gx, ghost_row_src<S, NX>(a, p, q, 2, z, y, nuz), rowb, &full[s]);
                 }
                 continue;
             }
@@ -482,25 +518,17 @@ __device__ void producer(const StepArgs &a, const TiledArgs &p, char *smem, uint
             if (it < nch) {
                 const int y = ya + it * p.chunk;
                 if (y < yb)
-                    bulk_g2s(slice + (size_t)(y - ybox0) * NX, e + pbase + ((long long)z * ny + y) * gx,
+                    bulk_g2s(slice + (size_t)(y - ybox0) * gx, e + pbase + ((long long)z * ny + y) * gx,
                              (uint32_t)min(p.chunk, yb - y) * rowb, &full[s]);
             } else if (it < nch + 4) {
                 const int g = it - nch;  // 0, 1: below the domain; 2, 3: above it
                 const int y = g < 2 ? ylo + g : yb + (g - 2);
                 if (g < 2 ? y < ya : y < yhi)
-                    bulk_g2s(slice + (size_t)(y - ybox0) * NX, ghost_row_src<S, NX>(a, p, q, 1, y, z, nuy), rowb, &full[s]);
+                    bulk_g2s(slice + (size_t)(y - ybox0) * gx, ghost_row_src<S, NX>(a, p, q, 1, y, z, nuy), rowb, &full[s]);
             }
         }
-        // x-wall ghosts outside the tile: 16 bytes of the mirrored direction's row (specular), or
-        // the diffuse values of the tile's rows (incoming directions only)
+        // x-wall ghosts outside the tile: the diffuse values of its rows (incoming directions only)
         for (int sd = 0; sd < 2; ++sd) {
-            if (spec[sd]) {
-                const long long mb = ((long long)q.k * a.nd + a.mirror[q.d]) * a.ncell + (sd ? gx - V : 0);
-                for (int j = lane; j < ncore; j += 32) {
-                    const int yl = j % q.nyt, zl = j / q.nyt;
-                    bulk_g2s(SD::spec(side, sd, zl, yl), e + mb + ((long long)(q.z0 + zl) * ny + q.y0 + yl) * gx, 16, &full[s]);
-                }
-            }
             if (dif[sd])
                 for (int zl = lane; zl < q.nzt; zl += 32) {
                     const long long s0 = dcol_src(a, sd, q.k, q.z0 + zl, q.y0);
@@ -534,13 +562,13 @@ __device__ void producer(const StepArgs &a, const TiledArgs &p, char *smem, uint
 
 // ---- consumer warps -----------------------------------------------------------------------
 // Where an end lane of a warp takes its two x-neighbours from (besides the plain shuffle).
-enum { kGhShfl = 0, kGhSmem = 1, kGhSpec = 2, kGhDiff = 3, kGhConst = 4, kGhOwn = 5 };
+enum { kGhShfl = 0, kGhSmem = 1, kGhConst = 4, kGhOwn = 5 };
 
 // SY, SX: signs of the direction's y and x components (+1 when positive, else -1), fixed per
 // instance so that row steps are constants and the x faces need no orientation branch.  FULL:
 // the warp's KR rows all lie in the tile (every tile but a ragged last one), so the row loop
 // carries no exit test.
-template <int S, int LIM, int VL, int WPR, int DIM, bool SR, int SY, int SX, bool FULL>
+template <int S, int LIM, int VL, int WPR, int DIM, bool SR, bool FR, int SY, int SX, bool FULL>
 __device__ __forceinline__ void rows_of_warp(const StepArgs &a, const TiledArgs &p, const PT &q, const char *stage,
                                              int zl, int rb, int half, float *accsm,
                                              float (&acc)[Geo<DIM, WPR>::KR][VL], const float *btsm, float *wsm,
@@ -549,7 +577,7 @@ __device__ __forceinline__ void rows_of_warp(const StepArgs &a, const TiledArgs 
     constexpr bool REF = St<S>::kRef;
     constexpr int NX = 32 * VL * WPR, TY = Geo<DIM, WPR>::TY, RY = TY + 4;
     const int lane = threadIdx.x & 31, x0 = (half * 32 + lane) * VL;
-    const int rowlen = a.n[0], ny = a.n[1], nz = a.n[2];
+    const int rowlen = FR ? NX : a.n[0], ny = a.n[1], nz = a.n[2];
     // The grid's rows hold rowlen <= NX cells (a multiple of VL): lanes past the row's end compute
     // on unused box columns and store nothing.  The right end lane of this warp's part of the row
     // holds its last cell (lane 31 unless the row ends inside this warp's part).
@@ -569,9 +597,10 @@ __device__ __forceinline__ void rows_of_warp(const StepArgs &a, const TiledArgs 
     const int zbox0 = DIM == 3 ? q.z0 - (sz > 0 ? 2 : 1) : 0;
     const int z = q.z0 + zl;
     const T *box = reinterpret_cast<const T *>(stage);
-    const int dy = sy * NX;                    // next row in streaming order (elements)
-    const int dz = sz * (TY + 3) * NX;         // next slice downwind (elements)
-    int o = ((z - zbox0) * (TY + 3) + (q.y0 + yl0 - ybox0)) * NX;  // row start in the box
+    const int dy = sy * rowlen;                // next row in streaming order (elements of the box)
+    const int dyt = sy * NX;                   // and of the tile arrays
+    const int dz = sz * (TY + 3) * rowlen;     // next slice downwind (elements)
+    int o = ((z - zbox0) * (TY + 3) + (q.y0 + yl0 - ybox0)) * rowlen;  // row start in the box
     int c = (zl * TY + yl0) * NX + x0;         // this lane's cells in the tile arrays
     // the same row in the reference box (rows y0-2.., slices z0-2..), and its upwind steps; a
     // second ghost layer of a thermalizing or diffuse wall holds the wall value coded against
@@ -628,11 +657,11 @@ __device__ __forceinline__ void rows_of_warp(const StepArgs &a, const TiledArgs 
             rx1 = gi + gi1;
         } else if (bc == kBcSpecular) {
             gptr = SD::spec(side, sd, zl, yl0);
-            gstep = sy * SD::V;
-            gi0 = sd == 0 ? 0 : SD::V - 1;
-            gi1 = sd == 0 ? 1 : SD::V - 2;
-            rx0 = (sd == 0 ? 0 : rowlen - SD::V) + gi0;
-            rx1 = (sd == 0 ? 0 : rowlen - SD::V) + gi1;
+            gstep = 2 * sy;
+            gi0 = sd == 0 ? 0 : 1;
+            gi1 = 1 - gi0;
+            rx0 = sd == 0 ? 0 : rowlen - 1;
+            rx1 = sd == 0 ? 1 : rowlen - 2;
         } else if (leaving) {
             gmode = kGhOwn;
             // FP32: read the lane's own end cell from the box row (same value, no select)
@@ -745,7 +774,7 @@ __device__ __forceinline__ void rows_of_warp(const StepArgs &a, const TiledArgs 
             #pragma unroll
             for (int v = 0; v < VL; ++v) ac[v] = accsm[c + v];
         }
-        typename St<S>::C h[VL];
+        typename St<S>::C h[code_words<S, VL>()];
         float en[VL], es[VL];
         const long long grow = ((long long)z * ny + y) * rowlen;  // global index of the row's first cell
         // FP32: e^{n+1} = e - dt/tau e + bt - |nu_y| (F_out - F_in) - nu_x (F_{v+1} - F_v)
@@ -770,11 +799,23 @@ __device__ __forceinline__ void rows_of_warp(const StepArgs &a, const TiledArgs 
             if constexpr (DIM == 3) t = fmaf(-anz, zo[v] - zi[v], t);
             en[v] = t;
         }
-        #pragma unroll
-        for (int v = 0; v < VL; ++v) {
-            if constexpr (SR) h[v] = St<S>::enc_sr(en[v], mix32(pkey ^ (uint32_t)(grow + x0 + v)));
-            else h[v] = St<S>::enc(en[v]);
-            es[v] = St<S>::val(h[v]);
+        if constexpr (!REF) {
+            #pragma unroll
+            for (int v = 0; v < VL; ++v) h[v] = es[v] = en[v];
+        } else {
+            #pragma unroll
+            for (int v = 0; v < VL; v += 2) {
+                const float nx2 = v + 1 < VL ? en[v + 1 < VL ? v + 1 : v] : 0.f;
+                if constexpr (SR) {
+                    h[v / 2] = St<S>::enc_sr(en[v], mix32(pkey ^ (uint32_t)(grow + x0 + v)));
+                    if (v + 1 < VL) h[v / 2] |= St<S>::enc_sr(nx2, mix32(pkey ^ (uint32_t)(grow + x0 + v + 1))) << 16;
+                } else {
+                    h[v / 2] = St<S>::enc2(make_float2(en[v], nx2));
+                }
+                const float2 q = St<S>::val2(h[v / 2]);
+                es[v] = q.x;
+                if (v + 1 < VL) es[v + 1 < VL ? v + 1 : v] = q.y;
+            }
         }
         // moment partials, two cells at a time
         #pragma unroll
@@ -829,7 +870,7 @@ __device__ __forceinline__ void rows_of_warp(const StepArgs &a, const TiledArgs 
             fin[v] = fout[v];
         }
         o += dy;
-        c += dy;
+        c += dyt;
         eo += dyg;
         ro += dyR;
     }
@@ -916,7 +957,7 @@ __device__ __forceinline__ void fill_ref_box(const StepArgs &a, const PT &q, flo
     }
 }
 
-template <int S, int LIM, int VL, int WPR, int DIM, bool SR>
+template <int S, int LIM, int VL, int WPR, int DIM, bool SR, bool FR>
 __device__ void consumer(const StepArgs &a, const TiledArgs &p, char *smem, uint64_t *full, uint64_t *empty) {
     constexpr bool REF = St<S>::kRef;
     constexpr int NX = 32 * VL * WPR, TY = Geo<DIM, WPR>::TY, NCW = Geo<DIM, WPR>::NCW;
@@ -924,7 +965,7 @@ __device__ void consumer(const StepArgs &a, const TiledArgs &p, char *smem, uint
     int zl, rb, half;
     warp_place<VL, WPR, DIM>(zl, rb, half);
     const int x0 = (half * 32 + lane) * VL;
-    const int gx = a.n[0], ny = a.n[1];
+    const int gx = FR ? 32 * VL * WPR : a.n[0], ny = a.n[1];
     float *wsm = reinterpret_cast<float *>(smem + p.wall_off);
     float *btsm = reinterpret_cast<float *>(smem + p.bt_off);
     float *accsm = reinterpret_cast<float *>(smem + p.acc_off);
@@ -934,6 +975,8 @@ __device__ void consumer(const StepArgs &a, const TiledArgs &p, char *smem, uint
         #pragma unroll
         for (int v = 0; v < VL; ++v) acc[r][v] = 0.f;
     float *rbox = reinterpret_cast<float *>(smem + p.rho_off);
+    // the specular x wall this lane is next to, -1: none
+    const int sside = x0 == 0 && a.bc[0] == kBcSpecular ? 0 : (x0 + VL == gx && a.bc[1] == kBcSpecular ? 1 : -1);
     int seg = -1, cur_unit = -1, cur_band = -1;
     int s = 0;         // stage of plane-tile i = i mod ns
     uint32_t ph = 0u;  // its use count parity = (i / ns) mod 2
@@ -983,6 +1026,18 @@ __device__ void consumer(const StepArgs &a, const TiledArgs &p, char *smem, uint
                 }
             }
         }
+        // the specular ghosts of the lanes next to an x wall, on their way while the warp waits
+        using Pair = typename std::conditional<St<S>::kRef, uint32_t, float2>::type;
+        Pair sg[Geo<DIM, WPR>::KR];
+        const bool mine = sside >= 0 && zl < q.nzt;
+        if (mine) {
+            const typename St<S>::T *m = static_cast<const typename St<S>::T *>(a.e_in) +
+                                         ((long long)q.k * a.nd + __ldg(a.mirror + q.d)) * a.ncell +
+                                         ((long long)(q.z0 + zl) * ny + q.y0 + rb) * gx + (sside == 0 ? 0 : gx - 2);
+            #pragma unroll
+            for (int r = 0; r < Geo<DIM, WPR>::KR; ++r)
+                if (rb + r < q.nyt) sg[r] = __ldg(reinterpret_cast<const Pair *>(m + (long long)r * gx));
+        }
         // warp-uniform: the stage's copies landed, else a bounded wait unless a warp gave up
         bool ok = __all_sync(0xffffffffu, mbar_try_wait(&full[s], ph));
         if (!ok) {
@@ -1004,10 +1059,17 @@ __device__ void consumer(const StepArgs &a, const TiledArgs &p, char *smem, uint
         const char *stage = smem + p.stage0 + (size_t)s * p.stage_bytes;
         if constexpr (REF) wsum += reinterpret_cast<const float *>(stage + p.hdr_off)[3];
         if (zl < q.nzt && rb < q.nyt) {
+            if (mine) {
+                Pair *sp = reinterpret_cast<Pair *>(Side<S, WPR, DIM>::spec(const_cast<char *>(stage) + p.side_off, sside, zl, rb));
+                #pragma unroll
+                for (int r = 0; r < Geo<DIM, WPR>::KR; ++r)
+                    if (rb + r < q.nyt) sp[r] = sg[r];
+                asm volatile("" ::: "memory");
+            }
             const float *hd = reinterpret_cast<const float *>(stage + p.hdr_off);
             const bool px = hd[0] > 0.f, py = hd[1] > 0.f;  // the signs rows_of_warp takes
             const bool full = rb + Geo<DIM, WPR>::KR <= q.nyt;
-#define BTE_ROWS(SY_, SX_, F_) rows_of_warp<S, LIM, VL, WPR, DIM, SR, SY_, SX_, F_>(a, p, q, stage, zl, rb, half, accsm, acc, btsm, wsm, rbox)
+#define BTE_ROWS(SY_, SX_, F_) rows_of_warp<S, LIM, VL, WPR, DIM, SR, FR, SY_, SX_, F_>(a, p, q, stage, zl, rb, half, accsm, acc, btsm, wsm, rbox)
             if (full) {
                 if (py) { if (px) BTE_ROWS(1, 1, true); else BTE_ROWS(1, -1, true); }
                 else { if (px) BTE_ROWS(-1, 1, true); else BTE_ROWS(-1, -1, true); }
@@ -1029,7 +1091,7 @@ __device__ void consumer(const StepArgs &a, const TiledArgs &p, char *smem, uint
 
 // SR: 16-bit codes rounded stochastically (a separate instance, so the round-to-nearest one
 // carries none of the hashing)
-template <int S, int LIM, int VL, int WPR, int DIM, bool SR>
+template <int S, int LIM, int VL, int WPR, int DIM, bool SR, bool FR>
 __global__ void __launch_bounds__((Geo<DIM, WPR>::NCW + kProducerWarps) * 32, 1) k_step_tiled(const StepArgs a, const TiledArgs p) {
     extern __shared__ __align__(128) char smem[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem);
@@ -1053,46 +1115,56 @@ __global__ void __launch_bounds__((Geo<DIM, WPR>::NCW + kProducerWarps) * 32, 1)
     const int warp = (int)(threadIdx.x >> 5);
     if (warp >= Geo<DIM, WPR>::NCW) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Geo<DIM, WPR>::RP));
-        if (warp == Geo<DIM, WPR>::NCW) producer<S, VL, WPR, DIM>(a, p, smem, full, empty);
+        if (warp == Geo<DIM, WPR>::NCW) producer<S, VL, WPR, DIM, FR>(a, p, smem, full, empty);
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(Geo<DIM, WPR>::RC));
-        consumer<S, LIM, VL, WPR, DIM, SR>(a, p, smem, full, empty);
+        consumer<S, LIM, VL, WPR, DIM, SR, FR>(a, p, smem, full, empty);
     }
 }
 
 typedef void (*StepKernel)(const StepArgs, const TiledArgs);
 
 // row capacity 64: VL 2, one warp per row; 96: VL 3, one warp; 128: VL 4, one warp; 256 (2-D
-// only): VL 4, two warps
-template <int S, int LIM, int DIM, bool SR>
-StepKernel pick_nx(int nx) {
-    if (nx == 64) return k_step_tiled<S, LIM, 2, 1, DIM, SR>;
-    if (nx == 96) return k_step_tiled<S, LIM, 3, 1, DIM, SR>;
-    if (nx == 128) return k_step_tiled<S, LIM, 4, 1, DIM, SR>;
+// only): VL 4, two warps.  FR: the grid's rows fill the capacity, so that the box's strides are constants
+// (as run-time values they cost the hot spot and the laser block 1 to 2 %).
+template <int S, int LIM, int DIM, bool SR, bool FR>
+StepKernel pick_nx(int cap) {
+    if (cap == 64) return k_step_tiled<S, LIM, 2, 1, DIM, SR, FR>;
+    if (cap == 96) return k_step_tiled<S, LIM, 3, 1, DIM, SR, FR>;
+    if (cap == 128) return k_step_tiled<S, LIM, 4, 1, DIM, SR, FR>;
     if constexpr (DIM == 2) {
-        if (nx == 256) return k_step_tiled<S, LIM, 4, 2, DIM, SR>;
+        if (cap == 256) return k_step_tiled<S, LIM, 4, 2, DIM, SR, FR>;
     }
     return nullptr;
 }
 
+// the instance's row capacity, and whether the grid's rows fill it
+struct Rows {
+    int cap;
+    bool full;
+};
+template <int S, int LIM, int DIM, bool SR>
+StepKernel pick_rows(Rows r) {
+    return r.full ? pick_nx<S, LIM, DIM, SR, true>(r.cap) : pick_nx<S, LIM, DIM, SR, false>(r.cap);
+}
 template <int S, int DIM, bool SR>
-StepKernel pick_instance(int lim, int nx) {
-    if (lim == kLimFirst) return pick_nx<S, kLimFirst, DIM, SR>(nx);
-    if (lim == kLimMinmod) return pick_nx<S, kLimMinmod, DIM, SR>(nx);
-    return pick_nx<S, kLimVanAlbada, DIM, SR>(nx);
+StepKernel pick_instance(int lim, Rows r) {
+    if (lim == kLimFirst) return pick_rows<S, kLimFirst, DIM, SR>(r);
+    if (lim == kLimMinmod) return pick_rows<S, kLimMinmod, DIM, SR>(r);
+    return pick_rows<S, kLimVanAlbada, DIM, SR>(r);
 }
 
 // one definition per instantiation unit (sr: stochastic rounding of 16-bit codes)
-StepKernel pick_f32_2d(int lim, int nx);
-StepKernel pick_f32_3d(int lim, int nx);
-StepKernel pick_f16_2d(int lim, int nx, bool sr);
-StepKernel pick_f16_3d(int lim, int nx, bool sr);
-StepKernel pick_bf16_2d(int lim, int nx, bool sr);
-StepKernel pick_bf16_3d(int lim, int nx, bool sr);
-StepKernel pick_f16sr_2d(int lim, int nx);
-StepKernel pick_f16sr_3d(int lim, int nx);
-StepKernel pick_bf16sr_2d(int lim, int nx);
-StepKernel pick_bf16sr_3d(int lim, int nx);
+StepKernel pick_f32_2d(int lim, Rows r);
+StepKernel pick_f32_3d(int lim, Rows r);
+StepKernel pick_f16_2d(int lim, Rows r, bool sr);
+StepKernel pick_f16_3d(int lim, Rows r, bool sr);
+StepKernel pick_bf16_2d(int lim, Rows r, bool sr);
+StepKernel pick_bf16_3d(int lim, Rows r, bool sr);
+StepKernel pick_f16sr_2d(int lim, Rows r);
+StepKernel pick_f16sr_3d(int lim, Rows r);
+StepKernel pick_bf16sr_2d(int lim, Rows r);
+StepKernel pick_bf16sr_3d(int lim, Rows r);
 
 }  // namespace tiled
 }  // namespace bte
