@@ -66,7 +66,8 @@ struct bte_ctx {
     // tiled-kernel plan
     TiledPlan plan;
     bool tiled = false;
-    // register-streaming plan of the grids the tiled kernel does not take
+    // register-streaming plan (FP32, 2-D and 3-D): the forward step of the grids the tiled kernel does not
+    // take and of those it takes but steps slower; precedes `tiled`, which then keeps the adjoint
     StreamPlan splan;
     bool streamed = false;
     // persistent single-CTA path (small 1-D FP32 problems): per-call source amplitudes
@@ -559,8 +560,14 @@ extern "C" bte_status bte_create(const bte_grid *grid, const bte_bands *bands, c
             return bail(BTE_EUNSUPPORTED);
         }
     }
-    if (!c->persist && !c->tiled) {
-        std::string why;  // not applicable: the generic kernel
+    // The tiled forward kernel is the faster one in 2-D and, in 3-D, where a lane holds 4 cells and nearly
+    // every lane does (its shorter 3-D rows leave 12 warps too little work to hide their latencies).  Us a
+    // step with its finalize, tiled / streaming: 128^2 x 64, 5 x 96 1725 / 2105, rows of 100 cells 1755 /
+    // 1577, of 96 1733 / 1586, of 64 1521 / 1122; 32^2 x 16, 40 x 96 924 / 421; in 2-D 256^2, 20 x 128 318 / 442,
+    // 128^2, 20 x 64 69 / 80, rows of 96 166 / 230, of 64 156 / 175, 200^2 296 / 284.
+    const bool tiled_faster = c->tiled && (c->dim == 2 || (c->plan.nx == 128 && c->n[0] >= 112));
+    if (!c->persist && !tiled_faster && !(c->tiled && c->kernel == BTE_KERNEL_TILED)) {
+        std::string why;  // not applicable: the tiled or the generic kernel
         c->streamed = stream_plan(c->dim, c->n, c->nb, c->nd, c->s.data(), c->bc, c->jump, c->storage, c->limiter,
                                   c->splan, why);
     }
@@ -633,7 +640,8 @@ extern "C" bte_status bte_create(const bte_grid *grid, const bte_bands *bands, c
         // moment partials: band-major rows for the generic passes, segment rows for the tiled one
         size_t np = (size_t)c->nb * c->ncell;
         if (c->tiled) np = std::max(np, (size_t)c->plan.G * c->plan.tcells);
-        if (c->streamed) np *= c->splan.nchunk;  // a row per part of a band's directions
+        // a row per part of a band's directions
+        if (c->streamed) np = std::max(np, (size_t)c->nb * c->splan.nchunk * (size_t)c->ncell);
         if ((st = dalloc(c, &c->P, np)) != BTE_OK) return bail(st);
     }
     for (int i = 0; i < 2; ++i)
@@ -821,7 +829,7 @@ constexpr int kGraphSteps = 32;
 
 static bool graph_eligible(const bte_ctx *c) {
     const bool sr = c->rounding == BTE_ROUND_STOCHASTIC && c->storage != BTE_STORE_F32;
-    return !c->persist && !c->has_amp && !sr && !c->prof && !(c->tiled && c->plan.stall);
+    return !c->persist && !c->has_amp && !sr && !c->prof && !(c->tiled && !c->streamed && c->plan.stall);
 }
 
 static bte_status step_graphs(bte_ctx *c, int chunks) {
@@ -944,12 +952,12 @@ extern "C" bte_status bte_interface(bte_ctx *a, int wa, bte_ctx *b, int wb, cons
 
 // The forward step's main kernel by the context's plan.
 static cudaError_t launch_forward(bte_ctx *c, const StepArgs &a, cudaStream_t strm) {
+    if (c->streamed) return launch_step_stream(a, c->splan, strm);
     if (c->tiled) {
         const cudaError_t e = launch_step_tiled(a, c->plan, strm);
         c->plan.stall = 0;
         return e;
     }
-    if (c->streamed) return launch_step_stream(a, c->splan, strm);
     if (c->dim == 1) return launch_step_1d(a, c->storage, c->limiter, strm);
     return launch_step_generic(a, c->storage, c->limiter, strm);
 }
@@ -976,8 +984,8 @@ static bte_status step_one(bte_ctx *c, cudaStream_t strm) {
         // T_L^{n+1} goes to the buffer of the old code reference; T_L^n becomes the reference of
         // the new state
         float *TL_next = c->R;
-        if (c->tiled) e = launch_finalize_tiled(a, c->plan, c->storage, TL_next, strm);
-        else if (c->streamed) e = launch_finalize_stream(a, c->splan, TL_next, strm);
+        if (c->streamed) e = launch_finalize_stream(a, c->splan, TL_next, strm);
+        else if (c->tiled) e = launch_finalize_tiled(a, c->plan, c->storage, TL_next, strm);
         else if (c->dim == 1) e = launch_finalize_1d(a, c->storage, TL_next, strm);
         else e = launch_finalize(a, c->G, TL_next, strm);
         if (e != cudaSuccess) return fail(c, BTE_ECUDA, "finalize launch: %s", cudaGetErrorString(e));

@@ -135,10 +135,11 @@ bool stream_plan(int dim, const int n[3], int nb, int nd, const double *s, const
     plan.mixed = dim == 3;
     // Parts of a band's directions: enough blocks to fill the GPU many times over (in 3-D also short ones,
     // so that the slow blocks leave no tail), but no more than a row of moment partials (4 bytes a cell
-    // written and read) for every 12 directions where the blocks suffice.
+    // written and read) for every 12 directions where the blocks suffice, 4 where they then give every SM 8.
     const long long have = blocks * nb, want = (dim == 3 ? 64LL : 16LL) * sms, least = 4LL * sms;
     int nc = 1;
     while (have * nc < want && nd / (2 * nc) >= 12) nc *= 2;
+    while (have * nc < 2 * least && nd / (2 * nc) >= 4) nc *= 2;
     while (have * nc < least && nc < nd) nc *= 2;
     plan.nchunk = nc = std::min(nc, nd);
     if (blocks * nb * nc > INT_MAX) {
