@@ -6,6 +6,7 @@
 #include <cuda_fp16.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "bte_device.cuh"
 
@@ -145,6 +146,17 @@ __global__ void __launch_bounds__(256) k_moment_only(const StepArgs a) {
     store_iso_codes<Cd>(a, k, i, c, rho_i, b);
 }
 
+// A stored value, each operation rounded by itself: in straight-line code the compiler may fuse the scale
+// into the value's use, which the generic step's branches kept apart, and a code next to a rounding boundary
+// would differ.
+template <class Cd>
+__device__ __forceinline__ float ld_rn(const typename Cd::T *p, long long i, const BandConst &b, float rho) {
+    if constexpr (!Cd::kRef) return p[i];
+    else if constexpr (std::is_same<typename Cd::T, __half>::value)
+        return __fmul_rn(b.scale, __fadd_rn(__half2float(p[i]), rho));
+    else return __fmul_rn(b.scale, __fadd_rn(__bfloat162float(p[i]), rho));
+}
+
 // The 1-D step as two launches, a thread a (cell, direction) and the sums apart: the generic step's
 // threads each loop over their directions, 125 blocks on the grating's 1000 cells, and wait for one
 // value after another.  Same operations on the same values, and the sums in the generic step's order
@@ -163,14 +175,14 @@ __global__ void __launch_bounds__(256) k_step_1d(const StepArgs a) {
     const float eq = b.ck * a.TL[i];
     const float rho_new = rho_at<Cd>(a.TL, a.invTs, i);
     const float src = a.Q ? b.srck * (a.amp * a.Q[i]) : 0.f;
-    const float e0 = Cd::ld(ein, base + i, b, rho_at<Cd>(a.R, a.invTs, i));
+    const float e0 = ld_rn<Cd>(ein, base + i, b, rho_at<Cd>(a.R, a.invTs, i));
     const float nu = a.nu[plane * 3];
     float div = 0.f;
     if (nu != 0.f) {
         const int sg = nu > 0.f ? 1 : -1;
         float um2, um1, up1;
         if (i >= 2 && i + 2 < a.n[0]) {
-            auto at = [&](int j) { return Cd::ld(ein, base + j, b, rho_at<Cd>(a.R, a.invTs, j)); };
+            auto at = [&](int j) { return ld_rn<Cd>(ein, base + j, b, rho_at<Cd>(a.R, a.invTs, j)); };
             um2 = at(i - 2 * sg);
             um1 = at(i - sg);
             up1 = at(i + sg);
@@ -210,7 +222,7 @@ __global__ void __launch_bounds__(256) k_finalize_1d(const StepArgs a, float *TL
             #pragma unroll 8
             for (int d = grp; d < a.nd; d += ng) {
                 const int plane = k * a.nd + d;
-                const float es = Cd::ld(e, (long long)plane * a.ncell + i, b, rho);
+                const float es = ld_rn<Cd>(e, (long long)plane * a.ncell + i, b, rho);
                 acc += a.wmom[plane] * es;
                 if (wall >= 0) wacc += a.wdiff[wall * a.nd + d] * es;
             }
