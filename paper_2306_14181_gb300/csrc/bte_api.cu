@@ -1412,11 +1412,14 @@ struct AdjWork {
     bte_ctx *c;
     size_t ediff_bytes = 0;
     std::vector<void *> blocks;  // every device allocation of the call
-    ~AdjWork() {
-        for (void *p : blocks) cudaFree(p);
-    }
-    bool alloc(void **p, size_t bytes) {
-        if (cudaMalloc(p, bytes ? bytes : 16) != cudaSuccess) {
+    // small requests share allocations of kSlab bytes (an allocation and its release cost tens of
+    // microseconds each, and a call makes up to a hundred requests)
+    static constexpr size_t kSlab = (size_t)64 << 20, kSmall = (size_t)8 << 20;
+    char *slab = nullptr;
+    size_t slab_used = 0, slab_block = 0;
+    ~AdjWork() { release(0); }
+    bool alloc_block(void **p, size_t bytes) {
+        if (cudaMalloc(p, bytes) != cudaSuccess) {
             cudaGetLastError();
             *p = nullptr;
             return false;
@@ -1424,9 +1427,35 @@ struct AdjWork {
         blocks.push_back(*p);
         return true;
     }
-    bool snap(Snap &s) {
-        return alloc(&s.e, c->state_bytes) && alloc((void **)&s.R, c->ncell * sizeof(float)) &&
-               alloc((void **)&s.TL, c->ncell * sizeof(float)) && alloc(&s.ediff, ediff_bytes);
+    static size_t padded(size_t bytes) { return (std::max<size_t>(bytes, 16) + 255) / 256 * 256; }
+    bool alloc(void **p, size_t bytes) {
+        bytes = padded(bytes);
+        if (bytes > kSmall) return alloc_block(p, bytes);
+        if (!slab || slab_used + bytes > kSlab) {
+            void *q = nullptr;
+            if (!alloc_block(&q, kSlab)) return alloc_block(p, bytes);
+            slab = static_cast<char *>(q);
+            slab_used = 0;
+            slab_block = blocks.size() - 1;
+        }
+        *p = slab + slab_used;
+        slab_used += bytes;
+        return true;
+    }
+    void release(size_t mark) {  // the allocations after the first `mark`
+        if (slab && slab_block >= mark) slab = nullptr;
+        for (size_t j = mark; j < blocks.size(); ++j) cudaFree(blocks[j]);
+        blocks.resize(mark);
+    }
+    bool snap(Snap &s) {  // one block: the state, its reference, T_L, the wall values
+        const size_t es = padded(c->state_bytes), fs = padded(c->ncell * sizeof(float));
+        char *q = nullptr;
+        if (!alloc((void **)&q, es + 2 * fs + padded(ediff_bytes))) return false;
+        s.e = q;
+        s.R = reinterpret_cast<float *>(q + es);
+        s.TL = reinterpret_cast<float *>(q + es + fs);
+        s.ediff = q + es + 2 * fs;
+        return true;
     }
 };
 
@@ -1497,8 +1526,9 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
     Snap fin;
     for (auto &s : L1)
         if (!w.snap(s)) return fail(c, BTE_ENOMEM, "adjoint checkpoints do not fit in device memory");
+    // (one level: the first state of a segment is its checkpoint)
     for (auto &s : L2)
-        if (!w.snap(s)) return fail(c, BTE_ENOMEM, "adjoint checkpoints do not fit in device memory");
+        if ((K2 > 1 || &s != &L2[0]) && !w.snap(s)) return fail(c, BTE_ENOMEM, "adjoint checkpoints do not fit in device memory");
     for (auto &s : L3)
         if (!w.snap(s)) return fail(c, BTE_ENOMEM, "adjoint checkpoints do not fit in device memory");
     if (!w.snap(fin)) return fail(c, BTE_ENOMEM, "adjoint checkpoints do not fit in device memory");
@@ -1610,11 +1640,16 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
     };
     bte_status st = BTE_OK;
     auto run = [&]() -> bte_status {
-        // forward sweep, keeping the segment checkpoints
+        // forward sweep, keeping the segment checkpoints, and of the last segment every state
         base_step = c->step;
         for (int s = 0; s < nseg; ++s) {
             TRY(snap_save(c, L1[s], w.ediff_bytes));
-            TRY(timed_steps(std::min(K, nsteps - s * K)));
+            const int n = std::min(K, nsteps - s * K), keep = K2 == 1 && s == nseg - 1 ? n : 1;
+            for (int m = 1; m < keep; ++m) {
+                TRY(timed_steps(1));
+                TRY(snap_save(c, L2[m], w.ediff_bytes));
+            }
+            TRY(timed_steps(n - keep + 1));
         }
         TRY(snap_save(c, fin, w.ediff_bytes));
         // J = sum p T_L^N and lambda^N
@@ -1639,16 +1674,23 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
         // reverse sweep, segment by segment
         for (int s = nseg - 1; s >= 0; --s) {
             const int n0 = s * K, n1 = std::min(nsteps, n0 + K);
+            if (K2 == 1) {
+                if (s < nseg - 1) {
+                    TRY(snap_restore(c, L1[s], w.ediff_bytes));
+                    for (int m = 1; m < n1 - n0; ++m) {
+                        TRY(timed_steps(1));
+                        TRY(snap_save(c, L2[m], w.ediff_bytes));
+                    }
+                }
+                for (int m = n1 - 1; m >= n0; --m) TRY(adj_step(m == n0 ? L1[s] : L2[m - n0]));
+                continue;
+            }
             TRY(snap_restore(c, L1[s], w.ediff_bytes));
             const int ns2 = (n1 - n0 + K2 - 1) / K2;
             for (int m = n0; m < n1; ++m) {
                 if ((m - n0) % K2 == 0) TRY(snap_save(c, L2[(m - n0) / K2], w.ediff_bytes));
-                if ((m - n0) / K2 == ns2 - 1 && K2 > 1) break;  // the last sub-checkpoint is taken
+                if ((m - n0) / K2 == ns2 - 1) break;  // the last sub-checkpoint is taken
                 if (m < n1 - 1) TRY(timed_steps(1));
-            }
-            if (K2 == 1) {
-                for (int m = n1 - 1; m >= n0; --m) TRY(adj_step(L2[m - n0]));
-                continue;
             }
             for (int sub = ns2 - 1; sub >= 0; --sub) {
                 const int m0 = n0 + sub * K2, m1 = std::min(n1, m0 + K2);
