@@ -219,12 +219,23 @@ __global__ void __launch_bounds__(256) k_finalize_1d(const StepArgs a, float *TL
         const BandConst b = a.band[k];
         float acc = 0.f, wacc = 0.f;
         if (valid) {
-            #pragma unroll 8
-            for (int d = grp; d < a.nd; d += ng) {
-                const int plane = k * a.nd + d;
-                const float es = ld_rn<Cd>(e, (long long)plane * a.ncell + i, b, rho);
-                acc += a.wmom[plane] * es;
-                if (wall >= 0) wacc += a.wdiff[wall * a.nd + d] * es;
+            // kBatch loads in flight together, the last ones too
+            constexpr int kBatch = 16;
+            for (int q = grp; q < a.nd; q += kBatch * ng) {
+                float es[kBatch], wm[kBatch];
+                #pragma unroll
+                for (int m = 0; m < kBatch; ++m) {
+                    const int d = min(q + m * ng, a.nd - 1), plane = k * a.nd + d;
+                    es[m] = ld_rn<Cd>(e, (long long)plane * a.ncell + i, b, rho);
+                    wm[m] = a.wmom[plane];
+                }
+                #pragma unroll
+                for (int m = 0; m < kBatch; ++m) {
+                    const int d = q + m * ng;
+                    if (d >= a.nd) break;
+                    acc += wm[m] * es[m];
+                    if (wall >= 0) wacc += a.wdiff[wall * a.nd + d] * es[m];
+                }
             }
         }
         if (ng > 1) {
