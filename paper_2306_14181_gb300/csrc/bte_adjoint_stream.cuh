@@ -21,8 +21,7 @@
 // What bounds it: issue and the FMA pipe (58 and 57 % busy, 16 warps an SM), 166 thread instructions an update
 // in 3-D, 91 in 2-D.  A launch, against the tiled step (k_adj_tiled, whose blocks stage a box, wait, and
 // exchange z faces between barriers): 96^3, 32 x 96, FP16 40.6 -> 19.2 ms (floor at the copy rate 4.0); 128^2,
-// 20 x 64, FP32 107 -> 92 us (37); against the generic one, a call with its forward steps: 115^2, 7 x 128
-// 18.7 -> 5.6 ms.
+// 20 x 64, FP32 107 -> 92 us (37).
 #pragma once
 
 #include "bte_adjoint.h"
@@ -80,12 +79,14 @@ template <int S, bool VEC> __device__ __forceinline__ float2 lde(const typename 
 constexpr float kTiny = 1e-30f;
 __device__ __forceinline__ float2 square(float2 a) { return __ffma2_rn(a, a, f2(0.5f * kTiny)); }
 template <int LIM>
-__device__ __forceinline__ void grads(float2 a, float2 sa, float2 b, float2 sb, float2 th, float2 &U, float2 &V) {
+__device__ __forceinline__ void grads(float2 a, float2 sa, float2 b, float2 sb, float2 th, bool up, float2 &U, float2 &V) {
     if constexpr (LIM == kLimFirst) {
         U = V = f2(0.f);
     } else if constexpr (LIM == kLimMinmod) {
         const float2 ab = __fmul2_rn(a, b);
-        const bool pa0 = fabsf(a.x) < fabsf(b.x), pa1 = fabsf(a.y) < fabsf(b.y);
+        // equal slopes: the downwind one counts
+        const bool pa0 = up ? fabsf(a.x) < fabsf(b.x) : fabsf(a.x) <= fabsf(b.x);
+        const bool pa1 = up ? fabsf(a.y) < fabsf(b.y) : fabsf(a.y) <= fabsf(b.y);
         const float t0 = ab.x > 0.f ? th.x : 0.f, t1 = ab.y > 0.f ? th.y : 0.f;
         U = make_float2(pa0 ? t0 : 0.f, pa1 ? t1 : 0.f);
         V = make_float2(pa0 ? 0.f : t0, pa1 ? 0.f : t1);
@@ -231,9 +232,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_adj_stream(const __grid_constan
                 dn = sub2(wn, w);
                 sn = square(dn);
                 float2 dead;
-                grads<LIM>(dm, square(dm), d0_, s0_, __fmul2_rn(f2(hy * myA), sub2(q0, qm)), dead, Vp);
+                grads<LIM>(dm, square(dm), d0_, s0_, __fmul2_rn(f2(hy * myA), sub2(q0, qm)), uy, dead, Vp);
                 th = __fmul2_rn(f2(hy * my0), sub2(qn, q0));
-                grads<LIM>(d0_, s0_, dn, sn, th, U, V);
+                grads<LIM>(d0_, s0_, dn, sn, th, uy, U, V);
             }
             float2 s2d = f2(0.f);
             #pragma unroll
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_adj_stream(const __grid_constan
                     const float2 db = sub2(wnn, wn), sb = square(db);
                     const float2 tn = __fmul2_rn(f2(j + 1 == kRows - 1 ? hy * my1 : (j + 1 == kRows ? hy * myB : hy)), sub2(qnn, qn));
                     float2 Un, Vn;
-                    grads<LIM>(dn, sn, db, sb, tn, Un, Vn);
+                    grads<LIM>(dn, sn, db, sb, tn, uy, Un, Vn);
                     v = __fadd2_rn(v, __ffma2_rn(f2(sy), th, __fadd2_rn(sub2(U, V), sub2(Vp, Un))));
                     Vp = V;
                     th = tn;
@@ -270,8 +271,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_adj_stream(const __grid_constan
                     const float2 tA = __fmul2_rn(hA, make_float2(ux ? t1 : t0, ux ? t2 : t1));
                     const float2 tB = __fmul2_rn(hB, make_float2(ux ? t3 : t2, ux ? t4 : t3));
                     float2 UA, VA, UB, VB;
-                    grads<LIM>(a0, sa0, make_float2(a0.y, m1), make_float2(sa0.y, sm), tA, UA, VA);
-                    grads<LIM>(make_float2(m1, b1.x), make_float2(sm, sb1.x), b1, sb1, tB, UB, VB);
+                    grads<LIM>(a0, sa0, make_float2(a0.y, m1), make_float2(sa0.y, sm), tA, ux, UA, VA);
+                    grads<LIM>(make_float2(m1, b1.x), make_float2(sm, sb1.x), b1, sb1, tB, ux, UB, VB);
                     const float2 own = __ffma2_rn(f2(sx), make_float2(tA.y, tB.x), sub2(make_float2(UA.y, UB.x), make_float2(VA.y, VB.x)));
                     v = __fadd2_rn(v, __fadd2_rn(own, sub2(VA, UB)));
                 }
@@ -290,9 +291,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_adj_stream(const __grid_constan
                     const float2 d1 = sub2(e1, e0), d2 = sub2(w, e1), d3 = sub2(e3, w), d4 = sub2(e4, e3);
                     const float2 q2s = square(d2), q3s = square(d3);
                     float2 dead, Vz, Uz, Wz, Ud;
-                    grads<LIM>(d1, square(d1), d2, q2s, t0, dead, Vz);
-                    grads<LIM>(d2, q2s, d3, q3s, t1, Uz, Wz);
-                    grads<LIM>(d3, q3s, d4, square(d4), t2, Ud, dead);
+                    grads<LIM>(d1, square(d1), d2, q2s, t0, uz, dead, Vz);
+                    grads<LIM>(d2, q2s, d3, q3s, t1, uz, Uz, Wz);
+                    grads<LIM>(d3, q3s, d4, square(d4), t2, uz, Ud, dead);
                     v = __fadd2_rn(v, __ffma2_rn(f2(sz), t1, __fadd2_rn(sub2(Uz, Wz), sub2(Vz, Ud))));
                 }
                 if constexpr (VEC) __stcs(reinterpret_cast<float2 *>(out + o), v);

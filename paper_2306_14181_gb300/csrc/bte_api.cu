@@ -70,6 +70,11 @@ struct bte_ctx {
     // take and of those it takes but steps slower; precedes `tiled`, which then keeps the adjoint
     StreamPlan splan;
     bool streamed = false;
+    // within the adjoint of an FP32 minmod run: the forward steps and a fresh T_L by the tiled or generic
+    // kernels.  Minmod's gradient jumps where two slopes are equal, and a last-bit change of the states moves
+    // the gradients by 1e-4; the other limiters' gradients are continuous.
+    bool plain = false;
+    bool fresh = false;  // T_L was formed by refresh_moments, no step since
     // persistent single-CTA path (small 1-D FP32 problems): per-call source amplitudes
     bool persist = false;
     float *d_amp = nullptr;
@@ -328,7 +333,8 @@ static bte_status refresh_moments(bte_ctx *c) {
     a.e_in = c->e[c->cur];
     a.ediff_out = c->ediff[c->ecur ^ 1];
     c->ecur ^= 1;
-    if (c->storage == BTE_STORE_F32 && c->dim >= 2) {
+    c->fresh = true;
+    if (c->storage == BTE_STORE_F32 && c->dim >= 2 && !c->plain) {
         CU(c, launch_moment_rows(a, c->stream));
         CU(c, launch_tl_and_walls(a, c->nb, static_cast<const float *>(a.e_in), c->TL, c->stream));
     } else {
@@ -829,7 +835,7 @@ constexpr int kGraphSteps = 32;
 
 static bool graph_eligible(const bte_ctx *c) {
     const bool sr = c->rounding == BTE_ROUND_STOCHASTIC && c->storage != BTE_STORE_F32;
-    return !c->persist && !c->has_amp && !sr && !c->prof && !(c->tiled && !c->streamed && c->plan.stall);
+    return !c->persist && !c->has_amp && !sr && !c->prof && !c->plain && !(c->tiled && !c->streamed && c->plan.stall);
 }
 
 static bte_status step_graphs(bte_ctx *c, int chunks) {
@@ -889,6 +895,7 @@ extern "C" bte_status bte_step(bte_ctx *c, int nsteps) {
     if (c->peer) return fail(c, BTE_ESTATE, "the context is coupled at an interface: it steps through bte_step_pair");
     // after synthetic iterations the step starts from the state's own T_L (Eq. BTE_get_e0)
     if (c->tl_corrected && nsteps > 0) TRY(refresh_moments(c));
+    if (nsteps > 0) c->fresh = false;
     if (c->persist) return nsteps > 0 ? step_persistent(c, nsteps) : BTE_OK;
     int s = 0;
     if (nsteps >= 2 * kGraphSteps && graph_eligible(c)) {
@@ -952,7 +959,7 @@ extern "C" bte_status bte_interface(bte_ctx *a, int wa, bte_ctx *b, int wb, cons
 
 // The forward step's main kernel by the context's plan.
 static cudaError_t launch_forward(bte_ctx *c, const StepArgs &a, cudaStream_t strm) {
-    if (c->streamed) return launch_step_stream(a, c->splan, strm);
+    if (c->streamed && !c->plain) return launch_step_stream(a, c->splan, strm);
     if (c->tiled) {
         const cudaError_t e = launch_step_tiled(a, c->plan, strm);
         c->plan.stall = 0;
@@ -963,6 +970,7 @@ static cudaError_t launch_forward(bte_ctx *c, const StepArgs &a, cudaStream_t st
 }
 
 static bte_status step_one(bte_ctx *c, cudaStream_t strm) {
+    c->fresh = false;
     {
         StepArgs a = make_args(c);
         a.amp = (float)amplitude_at(c, c->step);
@@ -984,7 +992,7 @@ static bte_status step_one(bte_ctx *c, cudaStream_t strm) {
         // T_L^{n+1} goes to the buffer of the old code reference; T_L^n becomes the reference of
         // the new state
         float *TL_next = c->R;
-        if (c->streamed) e = launch_finalize_stream(a, c->splan, TL_next, strm);
+        if (c->streamed && !c->plain) e = launch_finalize_stream(a, c->splan, TL_next, strm);
         else if (c->tiled) e = launch_finalize_tiled(a, c->plan, c->storage, TL_next, strm);
         else if (c->dim == 1) e = launch_finalize_1d(a, c->storage, TL_next, strm);
         else e = launch_finalize(a, c->G, TL_next, strm);
@@ -1486,9 +1494,14 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
     if (nsteps < 0) return fail(c, BTE_EINVAL, "nsteps must be >= 0");
     if (ckpt_every < 0) return fail(c, BTE_EINVAL, "ckpt_every must be >= 0");
     if (c->peer) return fail(c, BTE_ESTATE, "the context is coupled at an interface (no adjoint of the pair)");
-    if (c->tl_corrected) TRY(refresh_moments(c));
     for (long long i = 0; i < c->ncell; ++i)
         if (!std::isfinite(probe[i])) return fail(c, BTE_EINVAL, "probe holds a non-finite value at cell %lld", i);
+    struct Plain {
+        bte_ctx *c;
+        ~Plain() { c->plain = false; }
+    } plain{c};
+    c->plain = c->limiter == BTE_LIM_MINMOD && c->storage == BTE_STORE_F32 && c->dim >= 2;
+    if (c->tl_corrected || (c->plain && c->fresh)) TRY(refresh_moments(c));
     const long long nc = c->ncell, nel = c->nelem;
     int K = ckpt_every > 0 ? ckpt_every : std::max(1, (int)std::ceil(std::sqrt((double)std::max(nsteps, 1))));
     K = std::max(1, std::min(K, std::max(nsteps, 1)));
@@ -1546,13 +1559,16 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
                 return false;
         return true;
     };
-    // The streaming step where it applies and its buffers fit; else the tiled step on rows that fill the
-    // forward kernel's row capacity exactly, else the generic one.
+    // The streaming step in the place of the tiled one (rows that fill the forward kernel's row capacity
+    // exactly) where it applies and its buffers fit; else the tiled step, else the generic one.  (On other
+    // grids it is two to three times faster than the generic step, but dJ/dlog tau, sums that cancel, then
+    // differs by up to 4e-5 from the generic step's, whose own error against 64 bits is 5e-5 there.)
     AdjStreamPlan ap;
     int dev = 0, sms = 0;
     CU(c, cudaGetDevice(&dev));
     CU(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    bool stream_adj = c->kernel == BTE_KERNEL_AUTO && adj_stream_plan(make_args(c), c->jump, sms, ap);
+    const bool full_rows = c->tiled && c->nd <= adj_walls_max_dirs() && c->plan.nx == c->n[0];
+    bool stream_adj = c->kernel == BTE_KERNEL_AUTO && full_rows && adj_stream_plan(make_args(c), c->jump, sms, ap);
     if (stream_adj) {
         const size_t mark = w.blocks.size(), rows = (size_t)c->nb * ap.nchunk;
         stream_adj = w.alloc((void **)&Pm, rows * nc * sizeof(float)) &&
@@ -1560,7 +1576,7 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
                      w.alloc((void **)&mtp, (size_t)adj_sfinal_blocks(nc) * sizeof(double)) && wall_buffers();
         if (!stream_adj) w.release(mark);
     }
-    const bool tiled_adj = !stream_adj && c->tiled && c->nd <= adj_walls_max_dirs() && c->plan.nx == c->n[0];
+    const bool tiled_adj = !stream_adj && full_rows;
     if (tiled_adj) {
         const size_t gt_rows = (size_t)std::max(1, c->plan.G);
         if (!w.alloc((void **)&Pm, gt_rows * c->plan.tcells * sizeof(float)) ||

@@ -146,12 +146,13 @@ def test_specular_x_and_short_rows_16bit(dim, n, bc, storage):
     assert np.max(np.abs(gTL - oTL)) / scale <= TOL16
 
 
-@pytest.mark.parametrize("dim,n,bc", [TILED[1], TILED[2], TILED[4]])
-def test_adjoint_after_the_default_forward(dim, n, bc):
-    """Grids whose forward steps stream and whose adjoint steps are tiled."""
-    from paper_2306_14181_gb300 import bte
-    cfg, P, ctx, Q, amps, dT0, p = _setup(dim, n, bc, 2, 0, 6)
-    assert ctx.info.kernel == bte.BTE_KERNEL_TILED
+@pytest.mark.parametrize("limiter", [0, 1, 2])
+@pytest.mark.parametrize("dim,n,bc", [TILED[1], TILED[2], TILED[4], (2, (37, 21, 1), [DIF, SPE, ISO, DIF, PER, PER]),
+                                      (2, (2, 4, 1), [PER, PER, SPE, DIF, PER, PER]),
+                                      (3, (13, 5, 2), [SPE, ISO, PER, PER, DIF, SPE])])
+def test_adjoint_by_default(dim, n, bc, limiter):
+    """The streaming adjoint, after tiled, streaming and (minmod) generic forward steps."""
+    cfg, P, ctx, Q, amps, dT0, p = _setup(dim, n, bc, limiter, 0, 6)
     J, gQ, gt = _gpu_adjoint(ctx, Q, amps, dT0, p, 6, ckpt=2)
     Jo, gQo, gto = P.adjoint(P.equilibrium(np.asarray(dT0, np.float32).astype(np.float64)), 6, p, Q, amps)
     assert abs(J - Jo) <= 1e-5 * abs(Jo)
