@@ -428,11 +428,8 @@ cudaError_t launch_persist_1d(const StepArgs &a, int limiter, int nsteps, const 
         t = (t + 31) / 32 * 32;
         return t > 1024 ? 1024 : (int)t;
     };
-    // The flat form takes what the padded rows do not fit (one band whose state nearly fills a CTA), and long
-    // rows: a share goes out as a remote store a cell and CTA, about four cycles each.  Us a step, rows / flat:
-    // 100 cells by 10 CTAs 2.0 / 3.1, 73 by 14 1.6 / 2.1, 292 by 12 15.2 / 6.9.
-    if ((long long)n * (nb < 16 ? nb : 16) <= 1200 &&
-        launch_cluster(rows, a, threads, [=](int C) { return row_layout(n, nd, (nb + C - 1) / C, C).floats * sizeof(float); },
+    // the flat form takes what the padded rows do not fit (one band whose state nearly fills a CTA)
+    if (launch_cluster(rows, a, threads, [=](int C) { return row_layout(n, nd, (nb + C - 1) / C, C).floats * sizeof(float); },
                        err, nsteps, amps, e_io, tl_out, ediff_out, s))
         return err;
     if (launch_cluster(flat, a, [](int) { return 1024; }, [&](int C) { return persist_smem(a, C); }, err, nsteps, amps,
