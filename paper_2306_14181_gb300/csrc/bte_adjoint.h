@@ -46,6 +46,7 @@ int adj_walls_max_dirs();  // directions the wall pass's combine phase holds in 
 // mu^n, dJ/dQ += amp q^n, dJ/dlog tau from the segment scalars (mt_part: ceil(ncell/256) doubles).
 // The tiled adjoint step on the forward plan's tiles and schedule: lambda^n (interior and
 // periodic faces), segment rows Pm, Pq ([G][tcells]) and Ps ([G][2]).
+bool adj_tiled_available(const TiledPlan &plan, int storage, int limiter);  // an instance for the plan's rows
 cudaError_t launch_adj_tiled(const StepArgs &a, const TiledPlan &plan, const float *lam_in, float *lam_out,
                              const float *mu_in, float *Pm, float *Pq, float *Ps, const float *w, int storage,
                              int limiter, cudaStream_t s);

@@ -5,12 +5,20 @@ namespace bte {
 
 using namespace tiled;
 
+static AdjKernel adj_pick(const TiledPlan &plan, int storage, int limiter) {
+    return storage == kStoreF32 ? adj_pick_f32(limiter, plan.nx, plan.dim)
+           : storage == kStoreF16 ? adj_pick_f16(limiter, plan.nx, plan.dim)
+                                  : adj_pick_bf16(limiter, plan.nx, plan.dim);
+}
+
+bool adj_tiled_available(const TiledPlan &plan, int storage, int limiter) {
+    return adj_pick(plan, storage, limiter) != nullptr;
+}
+
 cudaError_t launch_adj_tiled(const StepArgs &a, const TiledPlan &plan, const float *lam_in, float *lam_out,
                              const float *mu_in, float *Pm, float *Pq, float *Ps, const float *w, int storage,
                              int limiter, cudaStream_t s) {
-    AdjKernel k = storage == kStoreF32 ? adj_pick_f32(limiter, plan.nx, plan.dim)
-                  : storage == kStoreF16 ? adj_pick_f16(limiter, plan.nx, plan.dim)
-                                         : adj_pick_bf16(limiter, plan.nx, plan.dim);
+    AdjKernel k = adj_pick(plan, storage, limiter);
     if (!k) return cudaErrorInvalidConfiguration;
     const int ncw = plan.dim == 2 ? Geo<2, 1>::NCW : Geo<3, 1>::NCW;
     // accumulators of mu and of the source gradient and the block reduction; in 3-D the z-face

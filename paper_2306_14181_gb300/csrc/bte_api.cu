@@ -1581,7 +1581,8 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
                      w.alloc((void **)&mtp, (size_t)adj_sfinal_blocks(nc) * sizeof(double)) && wall_buffers();
         if (!stream_adj) w.release(mark);
     }
-    const bool tiled_adj = !stream_adj && full_rows;
+    // (64-cell rows have no tiled instance)
+    const bool tiled_adj = !stream_adj && full_rows && adj_tiled_available(c->plan, c->storage, c->limiter);
     if (tiled_adj) {
         const size_t gt_rows = (size_t)std::max(1, c->plan.G);
         if (!w.alloc((void **)&Pm, gt_rows * c->plan.tcells * sizeof(float)) ||

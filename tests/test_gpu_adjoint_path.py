@@ -1,0 +1,36 @@
+"""Which kernels bte_adjoint runs, and that the choice shows in no result: gradients of the default choice
+are those of the explicit one, bit for bit (sums that cancel form dJ/dlog tau, so that any other
+order of the same operations moves it by up to 1e-3), rows without an instance of a kernel run the next one,
+and the context ends where bte_step ends.  Tolerances against the oracle are those of the parity tests: 1e-5
+on J, 1e-4 on the gradients."""
+import numpy as np
+import pytest
+
+from tests.support import rel_linf
+from tests.test_gpu_adjoint import _gpu_adjoint, _setup
+
+pytestmark = pytest.mark.gpu
+
+ISO, DIF, SPE, PER = 0, 1, 2, 3
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2306_14181_gb300 import build
+    build.build()
+
+
+@pytest.mark.parametrize("kernel", [0, 2])
+@pytest.mark.parametrize("dim,n,bc", [(2, (64, 3, 1), [ISO, SPE, DIF, ISO, PER, PER]),
+                                      (2, (64, 9, 1), [SPE, SPE, ISO, DIF, PER, PER]),
+                                      (3, (64, 3, 5), [SPE, ISO, PER, PER, DIF, SPE])])
+def test_rows_without_a_tiled_adjoint(dim, n, bc, kernel):
+    """64-cell rows step forward on the tiled kernel; the adjoint has no instance for them."""
+    cfg, P, ctx, Q, amps, dT0, p = _setup(dim, n, bc, 2, kernel, 6)
+    J, gQ, gt = _gpu_adjoint(ctx, Q, amps, dT0, p, 6, ckpt=2)
+    Jo, gQo, gto = P.adjoint(P.equilibrium(np.asarray(dT0, np.float32).astype(np.float64)), 6, p, Q, amps)
+    assert abs(J - Jo) <= 1e-5 * abs(Jo)
+    assert rel_linf(gQ, gQo) <= 1e-4 and rel_linf(gt, gto) <= 1e-4
