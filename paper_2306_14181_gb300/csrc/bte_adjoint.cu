@@ -22,7 +22,6 @@
 
 #include "bte_device.cuh"
 #include "bte_adjoint.h"
-#include "bte_adjoint_stream.cuh"
 
 namespace bte {
 
@@ -581,84 +580,19 @@ __global__ void __launch_bounds__(256) k_adj_tfinal(const StepArgs a, AdjTFinal 
     if (threadIdx.x == 0) mt_part[blockIdx.x] = sh[0];
 }
 
-// Finalize after the streaming adjoint: as k_adj_tfinal, from the parts' rows (row k nchunk + c holds
-// sum_d lambda^n of a part of band k's directions).  A block is 64 cells by 4 groups; group g takes rows
-// (and, of the wall corrections, bands) g, g + 4, ..., and group 0 adds the four sums in order.
-constexpr int kFinItems = 64, kFinGroups = 4;
-__global__ void __launch_bounds__(kFinItems * kFinGroups) k_adj_sfinal(const StepArgs a, AdjSFinal f, float amp,
-                                                                     float *mu_out, double *gQ, double *mt_part) {
-    __shared__ float pm[kFinGroups][kFinItems], pq[kFinGroups][kFinItems];
-    __shared__ double sh[kFinItems];
-    const int lane = threadIdx.x % kFinItems, grp = threadIdx.x / kFinItems;
-    const long long i = (long long)blockIdx.x * kFinItems + lane;
-    float m = 0.f, q = 0.f;
-    if (i < a.ncell) {
-        const int rows = a.nb * f.nchunk;
-        #pragma unroll 8
-        for (int r = grp; r < rows; r += kFinGroups) {
-            const float v = __ldcs(f.P + (long long)r * a.ncell + i);
-            const BandConst &b = a.band[r / f.nchunk];
-            m = fmaf(b.dtinv * b.ck, v, m);
-            q = fmaf(b.srck, v, q);
-        }
-        const int nx = a.n[0], ny = a.n[1];
-        const int c[3] = {(int)(i % nx), (int)((i / nx) % ny), (int)(i / ((long long)nx * ny))};
-        for (int ax = 0; ax < a.dim; ++ax) {
-            if (a.bc[2 * ax] == kBcPeriodic) continue;
-            const int n = a.n[ax], pos = c[ax];
-            if (pos >= 2 && pos < n - 2) continue;
-            const int o1 = ax == 0 ? 1 : 0, o2 = ax == 2 ? 1 : 2;
-            const long long nl = (long long)a.n[o1] * a.n[o2], line = (long long)c[o2] * a.n[o1] + c[o1];
-            const int sl = wall_slot(pos, n);
-            #pragma unroll 4
-            for (int k = grp; k < a.nb; k += kFinGroups) {
-                const float v = f.corr[ax][((long long)k * 4 + sl) * nl + line];
-                const BandConst &b = a.band[k];
-                m = fmaf(b.dtinv * b.ck, v, m);
-                q = fmaf(b.srck, v, q);
-            }
-        }
-    }
-    pm[grp][lane] = m;
-    pq[grp][lane] = q;
-    __syncthreads();
-    if (grp == 0) {
-        double mt = 0.0;
-        if (i < a.ncell) {
-            #pragma unroll
-            for (int g = 1; g < kFinGroups; ++g) {
-                m += pm[g][lane];
-                q += pq[g][lane];
-            }
-            mu_out[i] = m;
-            gQ[i] += (double)amp * (double)q;
-            mt = (double)f.mu_in[i] * (double)a.TL[i];
-        }
-        sh[lane] = mt;
-    }
-    __syncthreads();
-    for (int h = kFinItems / 2; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h) sh[threadIdx.x] += sh[threadIdx.x + h];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) mt_part[blockIdx.x] = sh[0];
-}
-
 // dJ/dlog tau_k += sum over band k's segments of (-dt/tau_k Ps0 - Ps1/(tau_k D))
 //                 + C_k/(tau_k D) sum_i mu^{n+1}_i T_L,i^n: one block per band, each thread a fixed
 // strided subset, then a fixed-order tree.
 constexpr int kTauThreads = 256;
-__global__ void __launch_bounds__(kTauThreads) k_adj_ttau(const StepArgs a, const float *Ps, const int *seg_band, int G,
-                                                          const double *mt_part, int nmt, double W, double *gtau) {
+__global__ void __launch_bounds__(kTauThreads) k_adj_ttau(const StepArgs a, AdjTFinal f, const double *mt_part, int nmt,
+                                                          double W, double *gtau) {
     __shared__ double sh[2][kTauThreads];
     const int k = blockIdx.x;
     const BandConst b = a.band[k];
     double s = 0.0, mt = 0.0;
-    // no seg_band: each band has G / nb segments, one after another
-    const int per = G / a.nb, g0 = seg_band ? 0 : k * per, g1 = seg_band ? G : g0 + per;
-    for (int g = g0 + threadIdx.x; g < g1; g += kTauThreads)
-        if (!seg_band || seg_band[g] == k)
-            s += -(double)b.dtinv * (double)Ps[2 * g] - (double)Ps[2 * g + 1] * (double)b.wtau * (double)a.invD;
+    for (int g = threadIdx.x; g < f.G; g += kTauThreads)
+        if (f.seg_band[g] == k)
+            s += -(double)b.dtinv * (double)f.Ps[2 * g] - (double)f.Ps[2 * g + 1] * (double)b.wtau * (double)a.invD;
     for (int j = threadIdx.x; j < nmt; j += kTauThreads) mt += mt_part[j];
     sh[0][threadIdx.x] = s;
     sh[1][threadIdx.x] = mt;
@@ -727,52 +661,8 @@ cudaError_t launch_adj_tfinal(const StepArgs &a, const AdjTFinal &f, float amp, 
                               double *mt_part, double W, double *gtau, cudaStream_t s) {
     const int nblk = (int)((a.ncell + 255) / 256);
     k_adj_tfinal<<<nblk, 256, 0, s>>>(a, f, amp, mu_out, gQ, mt_part);
-    k_adj_ttau<<<a.nb, kTauThreads, 0, s>>>(a, f.Ps, f.seg_band, f.G, mt_part, nblk, W, gtau);
+    k_adj_ttau<<<a.nb, kTauThreads, 0, s>>>(a, f, mt_part, nblk, W, gtau);
     return cudaGetLastError();
-}
-
-cudaError_t launch_adj_sfinal(const StepArgs &a, const AdjSFinal &f, float amp, float *mu_out, double *gQ,
-                              double *mt_part, double W, double *gtau, cudaStream_t s) {
-    const int nblk = (int)((a.ncell + kFinItems - 1) / kFinItems);
-    k_adj_sfinal<<<nblk, kFinItems * kFinGroups, 0, s>>>(a, f, amp, mu_out, gQ, mt_part);
-    k_adj_ttau<<<a.nb, kTauThreads, 0, s>>>(a, f.Ps, nullptr, a.nb * f.nchunk * f.blocks, mt_part, nblk, W, gtau);
-    return cudaGetLastError();
-}
-long long adj_sfinal_blocks(long long ncell) { return (ncell + kFinItems - 1) / kFinItems; }
-
-// ---- launch of the streaming adjoint step (kernels in bte_adjoint_stream.cuh) ---------------------
-bool adj_stream_plan(const StepArgs &a, const double *jump, int sms, AdjStreamPlan &p) {
-    p = AdjStreamPlan();
-    if (a.dim < 2 || a.n[1] < adjs::kRows || a.nd > adj_walls_max_dirs()) return false;
-    for (int ax = 0; ax < a.dim; ++ax)
-        if (jump[ax] != 0.0) return false;  // a periodic jump's ghosts are not plain wrapped cells
-    if (a.ncell > (1LL << 29)) return false;  // offsets within a plane are 32-bit
-    p.nys = (a.n[1] + adjs::kRows - 1) / adjs::kRows;
-    p.G = (a.n[0] + 1) / 2;
-    const long long blocks = ((long long)p.nys * a.n[2] * p.G + adjs::kThreads - 1) / adjs::kThreads;
-    // parts of a band's directions: enough blocks for four turns of two an SM, at least 8 directions each
-    // (a part costs a row of partials, 8 bytes a cell, and the references' setup)
-    while (blocks * a.nb * p.nchunk < 8LL * sms && a.nd / (2 * p.nchunk) >= 8) p.nchunk *= 2;
-    if (blocks * a.nb * p.nchunk > (1LL << 30)) return false;
-    p.blocks = (int)blocks;
-    return p.valid = true;
-}
-
-cudaError_t launch_adj_stream(const StepArgs &a, const AdjStreamPlan &p, const AdjArgs &g, float *P, float *Ps, int storage,
-                              int limiter, cudaStream_t s) {
-    adjs::AdjStreamArgs t;
-    t.lam_in = g.lam_in;
-    t.lam_out = g.lam_out;
-    t.mu_in = g.mu_in;
-    t.P = P;
-    t.Ps = Ps;
-    t.w = g.w;
-    t.nchunk = p.nchunk;
-    t.nys = p.nys;
-    t.G = p.G;
-    t.blocks = p.blocks;
-    if (storage == kStoreF32) return adjs::launch_f32(a, t, limiter, s);
-    return storage == kStoreF16 ? adjs::launch_f16(a, t, limiter, s) : adjs::launch_bf16(a, t, limiter, s);
 }
 
 template <int S>

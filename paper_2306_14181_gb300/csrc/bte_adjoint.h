@@ -50,24 +50,6 @@ bool adj_tiled_available(const TiledPlan &plan, int storage, int limiter);  // a
 cudaError_t launch_adj_tiled(const StepArgs &a, const TiledPlan &plan, const float *lam_in, float *lam_out,
                              const float *mu_in, float *Pm, float *Pq, float *Ps, const float *w, int storage,
                              int limiter, cudaStream_t s);
-// The streaming adjoint step (bte_adjoint_stream.cuh): lambda^n (interior and periodic faces), rows P
-// [nb nchunk][ncell] of sum_d lambda^n and scalars Ps [nb nchunk blocks][2]; then its finalize.
-struct AdjStreamPlan {
-    bool valid = false;
-    int nchunk = 1, nys = 0, G = 0, blocks = 0;  // parts of a band's directions; strips; pairs; blocks a part
-};
-bool adj_stream_plan(const StepArgs &a, const double *jump, int sms, AdjStreamPlan &p);
-cudaError_t launch_adj_stream(const StepArgs &a, const AdjStreamPlan &p, const AdjArgs &g, float *P, float *Ps, int storage,
-                              int limiter, cudaStream_t s);
-struct AdjSFinal {
-    const float *P, *Ps, *mu_in;
-    const float *corr[3];  // wall corrections per axis [nb][4][lines]
-    int nchunk, blocks;
-};
-// (mt_part: adj_sfinal_blocks(ncell) doubles)
-cudaError_t launch_adj_sfinal(const StepArgs &a, const AdjSFinal &f, float amp, float *mu_out, double *gQ,
-                              double *mt_part, double W, double *gtau, cudaStream_t s);
-long long adj_sfinal_blocks(long long ncell);
 cudaError_t launch_adj_tfinal(const StepArgs &a, const AdjTFinal &f, float amp, float *mu_out, double *gQ,
                               double *mt_part, double W, double *gtau, cudaStream_t s);
 

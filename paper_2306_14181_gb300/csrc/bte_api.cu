@@ -1429,8 +1429,10 @@ struct AdjWork {
     // microseconds each, and a call makes up to a hundred requests)
     static constexpr size_t kSlab = (size_t)64 << 20, kSmall = (size_t)8 << 20;
     char *slab = nullptr;
-    size_t slab_used = 0, slab_block = 0;
-    ~AdjWork() { release(0); }
+    size_t slab_used = 0;
+    ~AdjWork() {
+        for (void *p : blocks) cudaFree(p);
+    }
     bool alloc_block(void **p, size_t bytes) {
         if (cudaMalloc(p, bytes) != cudaSuccess) {
             cudaGetLastError();
@@ -1449,16 +1451,10 @@ struct AdjWork {
             if (!alloc_block(&q, kSlab)) return alloc_block(p, bytes);
             slab = static_cast<char *>(q);
             slab_used = 0;
-            slab_block = blocks.size() - 1;
         }
         *p = slab + slab_used;
         slab_used += bytes;
         return true;
-    }
-    void release(size_t mark) {  // the allocations after the first `mark`
-        if (slab && slab_block >= mark) slab = nullptr;
-        for (size_t j = mark; j < blocks.size(); ++j) cudaFree(blocks[j]);
-        blocks.resize(mark);
     }
     bool snap(Snap &s) {  // one block: the state, its reference, T_L, the wall values
         const size_t es = padded(c->state_bytes), fs = padded(c->ncell * sizeof(float));
@@ -1554,42 +1550,24 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
     float *Pm = nullptr, *Pq = nullptr, *Ps = nullptr, *corr[3] = {nullptr, nullptr, nullptr};
     double *mtp = nullptr;
     float *wscr = nullptr;
-    // wall scratch and corrections, and the partials of the streaming or the tiled step
-    auto wall_buffers = [&]() {
-        if (!w.alloc((void **)&wscr, (size_t)std::max(1LL, adj_walls_scratch_floats(make_args(c))) * sizeof(float)))
-            return false;
-        for (int ax = 0; ax < c->dim; ++ax)
-            if (c->bc[2 * ax] != BTE_BC_PERIODIC &&
-                !w.alloc((void **)&corr[ax], (size_t)c->nb * 4 * (nc / c->n[ax]) * sizeof(float)))
-                return false;
-        return true;
-    };
-    // The streaming step in the place of the tiled one (rows that fill the forward kernel's row capacity
-    // exactly) where it applies and its buffers fit; else the tiled step, else the generic one.  (On other
-    // grids it is two to three times faster than the generic step, but dJ/dlog tau, sums that cancel, then
-    // differs by up to 4e-5 from the generic step's, whose own error against 64 bits is 5e-5 there.)
-    AdjStreamPlan ap;
-    int dev = 0, sms = 0;
-    CU(c, cudaGetDevice(&dev));
-    CU(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const bool full_rows = c->tiled && c->nd <= adj_walls_max_dirs() && c->plan.nx == c->n[0];
-    bool stream_adj = c->kernel == BTE_KERNEL_AUTO && full_rows && adj_stream_plan(make_args(c), c->jump, sms, ap);
-    if (stream_adj) {
-        const size_t mark = w.blocks.size(), rows = (size_t)c->nb * ap.nchunk;
-        stream_adj = w.alloc((void **)&Pm, rows * nc * sizeof(float)) &&
-                     w.alloc((void **)&Ps, 2 * rows * ap.blocks * sizeof(float)) &&
-                     w.alloc((void **)&mtp, (size_t)adj_sfinal_blocks(nc) * sizeof(double)) && wall_buffers();
-        if (!stream_adj) w.release(mark);
-    }
-    // (64-cell rows have no tiled instance)
-    const bool tiled_adj = !stream_adj && full_rows && adj_tiled_available(c->plan, c->storage, c->limiter);
+    // The tiled adjoint takes rows that fill the forward kernel's row capacity exactly (rows of 64 cells have
+    // no instance).
+    const bool tiled_adj = c->tiled && c->nd <= adj_walls_max_dirs() && c->plan.nx == c->n[0] &&
+                           adj_tiled_available(c->plan, c->storage, c->limiter);
     if (tiled_adj) {
         const size_t gt_rows = (size_t)std::max(1, c->plan.G);
         if (!w.alloc((void **)&Pm, gt_rows * c->plan.tcells * sizeof(float)) ||
             !w.alloc((void **)&Pq, gt_rows * c->plan.tcells * sizeof(float)) ||
             !w.alloc((void **)&Ps, 2 * gt_rows * sizeof(float)) ||
-            !w.alloc((void **)&mtp, (size_t)((nc + 255) / 256) * sizeof(double)) || !wall_buffers())
+            !w.alloc((void **)&mtp, (size_t)((nc + 255) / 256) * sizeof(double)) ||
+            !w.alloc((void **)&wscr, (size_t)std::max(1LL, adj_walls_scratch_floats(make_args(c))) * sizeof(float)))
             return fail(c, BTE_ENOMEM, "adjoint buffers do not fit in device memory");
+        for (int ax = 0; ax < c->dim; ++ax) {
+            if (c->bc[2 * ax] == BTE_BC_PERIODIC) continue;
+            const long long lines = nc / c->n[ax];
+            if (!w.alloc((void **)&corr[ax], (size_t)c->nb * 4 * lines * sizeof(float)))
+                return fail(c, BTE_ENOMEM, "adjoint buffers do not fit in device memory");
+        }
     }
     {
         std::vector<float> pf(probe, probe + nc);
@@ -1640,20 +1618,7 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
         g.lam_out = lam[cur ^ 1];
         g.mu_in = mu[cur];
         if (prof) CU(c, cudaEventRecord(ev0, c->stream));
-        const float amp_prev = s.step > base_step ? (float)amplitude_at(c, s.step - 1) : 0.f;
-        if (stream_adj) {
-            // the order of the tiled step below
-            CU(c, launch_adj_stream(a, ap, g, Pm, Ps, c->storage, c->limiter, c->stream));
-            CU(c, launch_adj_walls(a, g, c->storage, c->limiter, lam[cur ^ 1], corr, wscr, c->stream));
-            AdjSFinal f;
-            f.P = Pm;
-            f.Ps = Ps;
-            f.mu_in = mu[cur];
-            for (int ax = 0; ax < 3; ++ax) f.corr[ax] = corr[ax];
-            f.nchunk = ap.nchunk;
-            f.blocks = ap.blocks;
-            CU(c, launch_adj_sfinal(a, f, amp_prev, mu[cur ^ 1], gQ, mtp, c->W, gt, c->stream));
-        } else if (tiled_adj) {
+        if (tiled_adj) {
             // interior and periodic faces on the tiles, then the faces next to each wall, then
             // mu^n, dJ/dQ (the q^n of lambda^n with the amplitude of step n-1) and dJ/dlog tau
             CU(c, launch_adj_tiled(a, c->plan, lam[cur], lam[cur ^ 1], mu[cur], Pm, Pq, Ps, c->wf, c->storage,
@@ -1672,6 +1637,7 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
             f.ty = c->plan.ty;
             f.tz = c->plan.tz;
             f.nty = c->plan.nty;
+            const float amp_prev = s.step > base_step ? (float)amplitude_at(c, s.step - 1) : 0.f;
             CU(c, launch_adj_tfinal(a, f, amp_prev, mu[cur ^ 1], gQ, mtp, c->W, gt, c->stream));
         } else {
             CU(c, launch_adj_step(a, g, c->storage, c->limiter, c->stream));
@@ -1716,9 +1682,9 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
             g.lam_in = nullptr;
             g.mu_in = nullptr;
             CU(c, launch_adj_init(a, g, c->storage, pr, c->stream));
-            // the streaming and tiled paths take dJ/dQ of step N-1 from q^N here; the generic step
-            // kernel takes it from lambda^{n+1} itself
-            const float amp_last = (stream_adj || tiled_adj) && nsteps > 0 ? (float)amplitude_at(c, c->step - 1) : 0.f;
+            // the tiled path takes dJ/dQ of step N-1 from q^N here; the generic step kernel
+            // takes it from lambda^{n+1} itself
+            const float amp_last = tiled_adj && nsteps > 0 ? (float)amplitude_at(c, c->step - 1) : 0.f;
             CU(c, launch_adj_reduce(a, g, amp_last, mu[cur], gQ, tpart, gt, c->stream));
         }
         // reverse sweep, segment by segment

@@ -34,3 +34,19 @@ def test_rows_without_a_tiled_adjoint(dim, n, bc, kernel):
     Jo, gQo, gto = P.adjoint(P.equilibrium(np.asarray(dT0, np.float32).astype(np.float64)), 6, p, Q, amps)
     assert abs(J - Jo) <= 1e-5 * abs(Jo)
     assert rel_linf(gQ, gQo) <= 1e-4 and rel_linf(gt, gto) <= 1e-4
+
+
+@pytest.mark.parametrize("storage", [0, 1, 2])
+@pytest.mark.parametrize("limiter", [0, 2])
+@pytest.mark.parametrize("dim,n,bc", [(2, (96, 9, 1), [SPE, SPE, ISO, DIF, PER, PER]),
+                                      (2, (128, 13, 1), [PER, PER, SPE, DIF, PER, PER]),
+                                      (2, (256, 6, 1), [DIF, SPE, PER, PER, PER, PER]),
+                                      (3, (128, 5, 6), [ISO, DIF, SPE, SPE, PER, PER]),
+                                      (3, (128, 10, 7), [SPE, SPE, PER, PER, DIF, ISO])])
+def test_default_gradients_are_the_tiled_ones(dim, n, bc, limiter, storage):
+    out = []
+    for kernel in (0, 2):
+        cfg, P, ctx, Q, amps, dT0, p = _setup(dim, n, bc, limiter, kernel, 6, storage=storage)
+        out.append(_gpu_adjoint(ctx, Q, amps, dT0, p, 6, ckpt=2))
+    assert out[0][0] == out[1][0]
+    assert np.array_equal(out[0][1], out[1][1]) and np.array_equal(out[0][2], out[1][2])
