@@ -305,7 +305,8 @@ __device__ __forceinline__ int wall_slot(int pos, int n) { return pos < 2 ? pos 
 // wall cell and the next cell of the same plane; j = 2, 3: adjoints of ghost layers 1 and 2.
 // A direction enters through one wall and leaves through the other: three faces, of which the leaving one
 // has no slope but at a specular wall (with the general ghost routine evaluated for nine values a launch on the 96^3
-// block, 32 x 96, took 1.36 ms, now 1.06; 128^2, 20 x 64 12 -> 11 us).
+// block, 32 x 96, took 1.36 ms, now 1.06; 128^2, 20 x 64 12 -> 11 us).  Its values are rounded as that routine
+// rounds them: dJ/dlog tau, sums that cancel, shows any other last bits (1.5e-4 on the block).
 constexpr int kWallThreads = 128;
 constexpr long long kWallLineThreads = 65536;  // (line, band) pairs from which phase 2 takes a thread each
 
@@ -344,15 +345,15 @@ __global__ void __launch_bounds__(kWallThreads) k_adj_walls_a(const StepArgs a, 
     if (bi != kBcPeriodic && nu != 0.f) {
         const int p0 = si ? n - 1 : 0, p1 = p0 + sg;
         const float r0 = rho(p0), r1 = rho(p1);
-        const float u0 = Cd::ld(e, base + i0 + p0 * st, b, r0), u1 = Cd::ld(e, base + i0 + p1 * st, b, r1);
+        const float u0 = ld_rn<Cd>(e, base + i0 + p0 * st, b, r0), u1 = ld_rn<Cd>(e, base + i0 + p1 * st, b, r1);
         float g1, g2;
         if (bi == kBcSpecular) {
-            g1 = Cd::ld(e, mbase + i0 + p0 * st, b, r0);
-            g2 = Cd::ld(e, mbase + i0 + p1 * st, b, r1);
+            g1 = ld_rn<Cd>(e, mbase + i0 + p0 * st, b, r0);
+            g2 = ld_rn<Cd>(e, mbase + i0 + p1 * st, b, r1);
         } else {
             g1 = g2 = bi == kBcIsothermal ? a.iso[wi * a.nb + k]
-                                          : Cd::ld(static_cast<const T *>(a.ediff_in),
-                                                   ((long long)wi * a.nb + k) * a.wc_max + wall_cell(a, ax, c), b, r0);
+                                          : ld_rn<Cd>(static_cast<const T *>(a.ediff_in),
+                                                      ((long long)wi * a.nb + k) * a.wc_max + wall_cell(a, ax, c), b, r0);
         }
         const float l0 = lam[p0 * st], l1 = lam[p1 * st];
         const float pa = anu * l0, pb = anu * (l1 - l0);
@@ -373,11 +374,11 @@ __global__ void __launch_bounds__(kWallThreads) k_adj_walls_a(const StepArgs a, 
     if (bo != kBcPeriodic && nu != 0.f) {
         const int q0 = so ? n - 1 : 0, q1 = q0 - sg;
         const float r0 = rho(q0);
-        const float um = Cd::ld(e, base + i0 + q0 * st, b, r0);
+        const float um = ld_rn<Cd>(e, base + i0 + q0 * st, b, r0);
         float La = 0.f, Lb = 0.f;
         if (bo == kBcSpecular) {
-            const float ul = Cd::ld(e, base + i0 + q1 * st, b, rho(q1));
-            lim_grad<LIM>(um - ul, Cd::ld(e, mbase + i0 + q0 * st, b, r0) - um, La, Lb);
+            const float ul = ld_rn<Cd>(e, base + i0 + q1 * st, b, rho(q1));
+            lim_grad<LIM>(um - ul, ld_rn<Cd>(e, mbase + i0 + q0 * st, b, r0) - um, La, Lb);
         }
         const float ph = -anu * lam[q0 * st];
         const float w[3] = {ph * (1.f + 0.5f * (La - Lb)), ph * (-0.5f * La), ph * (0.5f * Lb)};

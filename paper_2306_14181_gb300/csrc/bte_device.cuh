@@ -5,6 +5,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "bte_internal.h"
 
 namespace bte {
@@ -83,6 +85,17 @@ template <> struct Codec<kStoreBF16> {
         return b.scale * (__bfloat162float(h) + rho);
     }
 };
+
+// A stored value, each operation rounded by itself: in straight-line code the compiler may fuse the scale
+// into the value's use, which the branches of the ghost routine below keep apart, and what is formed from it
+// would have other last bits (a code next to a rounding boundary another value).
+template <class Cd>
+__device__ __forceinline__ float ld_rn(const typename Cd::T *p, long long i, const BandConst &b, float rho) {
+    if constexpr (!Cd::kRef) return p[i];
+    else if constexpr (std::is_same<typename Cd::T, __half>::value)
+        return __fmul_rn(b.scale, __fadd_rn(__half2float(p[i]), rho));
+    else return __fmul_rn(b.scale, __fadd_rn(__bfloat162float(p[i]), rho));
+}
 
 // Scaled code reference rho_j = R_j / T_scale of cell j (0 for FP32 storage, R untouched).
 template <class Cd>

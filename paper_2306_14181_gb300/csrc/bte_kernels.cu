@@ -6,7 +6,6 @@
 #include <cuda_fp16.h>
 
 #include <mutex>
-#include <type_traits>
 
 #include "bte_device.cuh"
 
@@ -144,17 +143,6 @@ __global__ void __launch_bounds__(256) k_moment_only(const StepArgs a) {
                wacc[j] * a.inv_den[w], b, rho_i);
     }
     store_iso_codes<Cd>(a, k, i, c, rho_i, b);
-}
-
-// A stored value, each operation rounded by itself: in straight-line code the compiler may fuse the scale
-// into the value's use, which the generic step's branches kept apart, and a code next to a rounding boundary
-// would differ.
-template <class Cd>
-__device__ __forceinline__ float ld_rn(const typename Cd::T *p, long long i, const BandConst &b, float rho) {
-    if constexpr (!Cd::kRef) return p[i];
-    else if constexpr (std::is_same<typename Cd::T, __half>::value)
-        return __fmul_rn(b.scale, __fadd_rn(__half2float(p[i]), rho));
-    else return __fmul_rn(b.scale, __fadd_rn(__bfloat162float(p[i]), rho));
 }
 
 // The 1-D step as two launches, a thread a (cell, direction) and the sums apart: the generic step's

@@ -50,3 +50,23 @@ def test_default_gradients_are_the_tiled_ones(dim, n, bc, limiter, storage):
         out.append(_gpu_adjoint(ctx, Q, amps, dT0, p, 6, ckpt=2))
     assert out[0][0] == out[1][0]
     assert np.array_equal(out[0][1], out[1][1]) and np.array_equal(out[0][2], out[1][2])
+
+
+# dJ/dlog tau (two bands) by (dimension, limiter, storage): the wall pass with every stored value rounded by
+# itself, as the general ghost routine forms them
+WALL_BITS = {
+    (2, 2, 1): ('-0x1.e5ccc4b97b2dcp-19', '-0x1.40b018d511635p-15'),
+    (2, 2, 2): ('-0x1.e5217e0565c43p-19', '-0x1.422e3a6622496p-15'),
+    (3, 1, 1): ('0x1.b143abb1d0bf3p-16', '0x1.ae105c2fe4c33p-15'),
+    (3, 1, 2): ('0x1.b1336a0abe11ap-16', '0x1.ad99317dff515p-15'),
+    (3, 2, 1): ('0x1.b1fcddc9a9e13p-16', '0x1.b76ae6124b1d8p-15'),
+    (3, 2, 2): ('0x1.b20796b0b0ca5p-16', '0x1.b7d99614000d9p-15'),
+}
+
+
+@pytest.mark.parametrize("dim,limiter,storage", sorted(WALL_BITS))
+def test_16bit_wall_pass_rounds_each_operation(dim, limiter, storage):
+    n, bc = {2: ((96, 9, 1), [SPE, SPE, ISO, DIF, PER, PER]), 3: ((96, 10, 7), [SPE, ISO, DIF, SPE, DIF, ISO])}[dim]
+    cfg, P, ctx, Q, amps, dT0, p = _setup(dim, n, bc, limiter, 2, 6, storage=storage)
+    _, _, gt = _gpu_adjoint(ctx, Q, amps, dT0, p, 6, ckpt=2)
+    assert tuple(float(x).hex() for x in gt) == WALL_BITS[dim, limiter, storage]
