@@ -336,11 +336,10 @@ static bte_status refresh_moments(bte_ctx *c) {
     c->fresh = true;
     if (c->storage == BTE_STORE_F32 && c->dim >= 2 && !c->plain) {
         CU(c, launch_moment_rows(a, c->stream));
-        CU(c, launch_tl_and_walls(a, c->nb, static_cast<const float *>(a.e_in), c->TL, c->stream));
     } else {
         CU(c, launch_moment_only(a, c->storage, c->stream));
-        CU(c, launch_finalize(a, c->nb, c->TL, c->stream));
     }
+    CU(c, launch_finalize(a, c->nb, c->TL, c->stream));
     c->tl_corrected = false;
     c->iface_pure = true;
     if (c->peer) TRY(iface_mix(c));

@@ -76,7 +76,7 @@ struct StepArgs {
 // Launchers (bte_kernels.cu).  All return the launch error (cudaGetLastError()).
 cudaError_t launch_fill(const StepArgs &a, int storage, const double *dT0, float *R_out, cudaStream_t s);
 cudaError_t launch_moment_only(const StepArgs &a, int storage, cudaStream_t s);
-cudaError_t launch_moment_rows(const StepArgs &a, cudaStream_t s);  // FP32: the partials alone, no wall values
+cudaError_t launch_moment_rows(const StepArgs &a, cudaStream_t s);  // the same of an FP32 state
 cudaError_t launch_step_generic(const StepArgs &a, int storage, int limiter, cudaStream_t s);
 // The 1-D step of any storage: the update, then T_L and the diffuse-wall values from e_out.
 cudaError_t launch_step_1d(const StepArgs &a, int storage, int limiter, cudaStream_t s);

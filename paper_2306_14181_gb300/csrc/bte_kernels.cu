@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "bte_device.cuh"
@@ -244,49 +245,72 @@ __global__ void __launch_bounds__(256) k_finalize_1d(const StepArgs a, float *TL
     if (valid && grp == 0) TL_out[i] = total * a.invD;
 }
 
-// T_L moment partials of an FP32 state without stepping (after an equilibrium fill, a state upload or a
-// sweep): P[k][i] = sum_d w_d e/tau_k.  Bound by DRAM: a thread takes VL neighbouring cells (16 bytes)
-// of every fourth direction with eight loads in flight, and the four direction groups of a block are
-// added in order.  256^2, 40 x 128 (1.34 GB): 693 us by k_moment_only, a thread a cell and band.  (1-D
-// and 16-bit states keep that one: their T_L seeds runs that show its last bits.)
+// k_moment_only for an FP32 state, with the same bits: every sum runs over the directions in order, because a
+// T_L with other last bits moves the gradients of a run that starts from it (dJ/dlog tau by up to 5e-5).
+// Bound by DRAM: the first tblocks blocks a band form the partials P[k][i] = sum_d w_d e/tau_k, a thread VL
+// neighbouring cells (16 bytes) of all directions with kMomBatch loads in flight; the others take a wall cell a
+// thread and form its diffuse-wall value.  256^2, 40 x 128 (1.34 GB): 693 us by k_moment_only; with
+// four direction groups a block, another order, 0.03 ms less than this.
+struct MomWalls {
+    int n, w[6];
+    int tblocks, wblocks;  // blocks of the partials; blocks a wall
+};
+constexpr int kMomBatch = 8;
 template <int VL>
-__global__ void __launch_bounds__(256) k_moment_rows(const StepArgs a) {
-    __shared__ float part[4][VL][64];
-    const int lane = threadIdx.x & 63, grp = threadIdx.x >> 6;
-    const long long i = ((long long)blockIdx.x * 64 + lane) * VL;
-    const bool valid = i < a.ncell;
+__global__ void __launch_bounds__(256) k_moment_rows(const __grid_constant__ StepArgs a,
+                                                     const __grid_constant__ MomWalls wl) {
     const int k = blockIdx.y;
+    const float *e = static_cast<const float *>(a.e_in) + (long long)k * a.nd * a.ncell;
+    if ((int)blockIdx.x >= wl.tblocks) {
+        const int q = blockIdx.x - wl.tblocks, wi = q / wl.wblocks, wall = wl.w[wi], ax = wall >> 1;
+        const long long j = (long long)(q - wi * wl.wblocks) * 256 + threadIdx.x;
+        const int n0 = ax == 0 ? a.n[1] : a.n[0], n1 = ax == 2 ? a.n[1] : a.n[2];
+        if (j >= (long long)n0 * n1) return;
+        const long long ja = j % n0, jb = j / n0, at = wall & 1 ? a.n[ax] - 1 : 0;
+        e += at * a.stride[ax] + ja * a.stride[ax == 0 ? 1 : 0] + jb * a.stride[ax == 2 ? 1 : 2];
+        const float *wd = a.wdiff + wall * a.nd;
+        float s = 0.f;
+        for (int d = 0; d < a.nd; d += kMomBatch) {
+            float f[kMomBatch];
+            #pragma unroll
+            for (int m = 0; m < kMomBatch; ++m) f[m] = __ldg(e + (long long)min(d + m, a.nd - 1) * a.ncell);
+            #pragma unroll
+            for (int m = 0; m < kMomBatch; ++m)
+                if (d + m < a.nd) s = fmaf(__ldg(wd + d + m), f[m], s);
+        }
+        static_cast<float *>(a.ediff_out)[((long long)wall * a.nb + k) * a.wc_max + j] = s * a.inv_den[wall];
+        return;
+    }
+    const long long i = ((long long)blockIdx.x * 256 + threadIdx.x) * VL;
+    if (i >= a.ncell) return;
+    const float *wm = a.wmom + (long long)k * a.nd;
+    float *P = a.P + (long long)k * a.ncell + i;
+    e += i;
     float s[VL];
     #pragma unroll
     for (int j = 0; j < VL; ++j) s[j] = 0.f;
-    if (valid) {
-        const float *e = static_cast<const float *>(a.e_in) + (long long)k * a.nd * a.ncell + i;
-        const float *wm = a.wmom + (long long)k * a.nd;
-        #pragma unroll 8
-        for (int d = grp; d < a.nd; d += 4) {
-            const float wd = __ldg(wm + d);
+    for (int d = 0; d < a.nd; d += kMomBatch) {
+        float f[kMomBatch][VL];
+        #pragma unroll
+        for (int m = 0; m < kMomBatch; ++m) {
+            const float *p = e + (long long)min(d + m, a.nd - 1) * a.ncell;
             if constexpr (VL == 4) {
-                const float4 f = __ldcs(reinterpret_cast<const float4 *>(e + (long long)d * a.ncell));
-                s[0] = fmaf(wd, f.x, s[0]);
-                s[1] = fmaf(wd, f.y, s[1]);
-                s[2] = fmaf(wd, f.z, s[2]);
-                s[3] = fmaf(wd, f.w, s[3]);
+                const float4 q = __ldcs(reinterpret_cast<const float4 *>(p));
+                f[m][0] = q.x; f[m][1] = q.y; f[m][2] = q.z; f[m][3] = q.w;
             } else {
-                s[0] = fmaf(wd, __ldcs(e + (long long)d * a.ncell), s[0]);
+                f[m][0] = __ldcs(p);
             }
         }
-    }
-    #pragma unroll
-    for (int j = 0; j < VL; ++j) part[grp][j][lane] = s[j];
-    __syncthreads();
-    if (grp == 0 && valid) {
         #pragma unroll
-        for (int j = 0; j < VL; ++j) {
+        for (int m = 0; m < kMomBatch; ++m) {
+            if (d + m >= a.nd) break;
+            const float wd = __ldg(wm + d + m);
             #pragma unroll
-            for (int g = 1; g < 4; ++g) s[j] += part[g][j][lane];
-            a.P[(long long)k * a.ncell + i + j] = s[j];
+            for (int j = 0; j < VL; ++j) s[j] = fmaf(wd, f[m][j], s[j]);
         }
     }
+    if constexpr (VL == 4) *reinterpret_cast<float4 *>(P) = make_float4(s[0], s[1], s[2], s[3]);
+    else *P = s[0];
 }
 
 // T_L_i = (sum_g P[g][i]) / sum_k C_k/tau_k, Eq. (BTE_get_e0), summed in fixed g order.
@@ -359,9 +383,21 @@ cudaError_t launch_moment_only(const StepArgs &a, int storage, cudaStream_t s) {
 }
 
 cudaError_t launch_moment_rows(const StepArgs &a, cudaStream_t s) {
+    MomWalls wl;
+    long long most = 0;
+    wl.n = 0;
+    for (int w = 0; w < 2 * a.dim; ++w) {
+        if (a.bc[w] != kBcDiffuse) continue;
+        wl.w[wl.n++] = w;
+        most = std::max(most, a.ncell / a.n[w >> 1]);
+    }
     // four cells a thread where planes are multiples of four cells (their loads are then aligned)
-    if (a.ncell % 4 == 0) k_moment_rows<4><<<dim3((unsigned)((a.ncell / 4 + 63) / 64), (unsigned)a.nb), 256, 0, s>>>(a);
-    else k_moment_rows<1><<<dim3((unsigned)((a.ncell + 63) / 64), (unsigned)a.nb), 256, 0, s>>>(a);
+    const bool quads = a.ncell % 4 == 0;
+    wl.tblocks = (int)(((quads ? a.ncell / 4 : a.ncell) + 255) / 256);
+    wl.wblocks = (int)((most + 255) / 256);
+    const dim3 g((unsigned)(wl.tblocks + wl.n * wl.wblocks), (unsigned)a.nb);
+    if (quads) k_moment_rows<4><<<g, 256, 0, s>>>(a, wl);
+    else k_moment_rows<1><<<g, 256, 0, s>>>(a, wl);
     return cudaGetLastError();
 }
 

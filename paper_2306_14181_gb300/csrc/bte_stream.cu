@@ -213,7 +213,7 @@ cudaError_t launch_step_stream(const StepArgs &a, const StreamPlan &plan, cudaSt
     return cudaGetLastError();
 }
 
-cudaError_t launch_tl_and_walls(const StepArgs &a, int rows, const float *state, float *TL_out, cudaStream_t s) {
+cudaError_t launch_finalize_stream(const StepArgs &a, const StreamPlan &plan, float *TL_out, cudaStream_t s) {
     WallList wl;
     wl.n = 0;
     wl.first[0] = 0;
@@ -226,12 +226,9 @@ cudaError_t launch_tl_and_walls(const StepArgs &a, int rows, const float *state,
     }
     const int tblocks = (int)((a.ncell + kItems - 1) / kItems);
     const unsigned blocks = (unsigned)tblocks + (unsigned)(wl.first[wl.n] / kItems) * (unsigned)a.nb;
-    k_finalize_stream<<<blocks, kItems * kGroups, 0, s>>>(a, rows, tblocks, wl, state, TL_out);
+    k_finalize_stream<<<blocks, kItems * kGroups, 0, s>>>(a, a.nb * plan.nchunk, tblocks, wl,
+                                                           static_cast<const float *>(a.e_out), TL_out);
     return cudaGetLastError();
-}
-
-cudaError_t launch_finalize_stream(const StepArgs &a, const StreamPlan &plan, float *TL_out, cudaStream_t s) {
-    return launch_tl_and_walls(a, a.nb * plan.nchunk, static_cast<const float *>(a.e_out), TL_out, s);
 }
 
 }  // namespace bte

@@ -41,9 +41,8 @@ bool stream_plan(int dim, const int n[3], int nb, int nd, const double *s, const
 bool stream_setup(StreamPlan &plan, std::string &why);
 void stream_free(StreamPlan &plan);
 cudaError_t launch_step_stream(const StepArgs &a, const StreamPlan &plan, cudaStream_t s);
-// T_L from `rows` rows of moment partials and the diffuse-wall values (a.ediff_out) of an FP32 state, in
-// one launch; and the same of the step a plan's forward launch took.
-cudaError_t launch_tl_and_walls(const StepArgs &a, int rows, const float *state, float *TL_out, cudaStream_t s);
+// T_L from the rows of moment partials and the diffuse-wall values (a.ediff_out) of the state it wrote, in one
+// launch.
 cudaError_t launch_finalize_stream(const StepArgs &a, const StreamPlan &plan, float *TL_out, cudaStream_t s);
 
 }  // namespace bte
