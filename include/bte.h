@@ -298,7 +298,9 @@ bte_status bte_run_steady(bte_ctx *ctx, long long max_steps, int check_every, do
 /* Discrete adjoint (the exact transpose of the step; the paper has no adjoint) of
  *     J = sum_i probe_i T_L,i   after nsteps steps from the context's current state,
  * T_L of Eq. (BTE_get_e0).  Runs the nsteps forward steps (the context ends in the state
- * bte_step(ctx, nsteps) leaves), then the adjoint steps backward in time:
+ * bte_step(ctx, nsteps) leaves), then the adjoint steps backward in time.  Where bte_step runs the
+ * register-streaming kernel, J and the gradients are those of the same steps on the tiled or generic
+ * kernel, whose states differ from the end state's by rounding:
  *     lambda^N = dT_L/de^T probe,  lambda^n = J_n^T lambda^{n+1}
  * with J_n the step's Jacobian at e^n (limited upwind flux with the limiter's Jacobian,
  * transposed wall ghosts, relaxation and the T_L coupling).  States are recomputed from
@@ -313,7 +315,8 @@ bte_status bte_adjoint(bte_ctx *ctx, int nsteps, int ckpt_every, const double *p
 
 /* With tracing on (bte_profile), the last bte_adjoint's device time of its adjoint steps
  * (transposed step plus its reductions, adj_steps of them) and of its forward steps
- * (the first sweep and the recomputations, fwd_steps of them).  Any pointer may be NULL. */
+ * (the first sweep, the recomputations and the steps to the end state where bte_step streams,
+ * fwd_steps of them).  Any pointer may be NULL. */
 bte_status bte_adjoint_profile_read(bte_ctx *ctx, double *adj_ms, long long *adj_steps, double *fwd_ms,
                                     long long *fwd_steps);
 

@@ -70,11 +70,10 @@ struct bte_ctx {
     // take and of those it takes but steps slower; precedes `tiled`, which then keeps the adjoint
     StreamPlan splan;
     bool streamed = false;
-    // within the adjoint of an FP32 minmod run: the forward steps and a fresh T_L by the tiled or generic
-    // kernels.  Minmod's gradient jumps where two slopes are equal, and a last-bit change of the states moves
-    // the gradients by 1e-4; the other limiters' gradients are continuous.
+    // bte_adjoint sets it while it steps the trajectory it differentiates: tiled or generic steps where
+    // bte_step streams.  dJ/dlog tau is a sum that cancels, and a last-bit change of the states moves it by up
+    // to 1e-3 (minmod's gradient also jumps where two slopes are equal).
     bool plain = false;
-    bool fresh = false;  // T_L was formed by refresh_moments, no step since
     // persistent single-CTA path (small 1-D FP32 problems): per-call source amplitudes
     bool persist = false;
     float *d_amp = nullptr;
@@ -333,8 +332,7 @@ static bte_status refresh_moments(bte_ctx *c) {
     a.e_in = c->e[c->cur];
     a.ediff_out = c->ediff[c->ecur ^ 1];
     c->ecur ^= 1;
-    c->fresh = true;
-    if (c->storage == BTE_STORE_F32 && c->dim >= 2 && !c->plain) {
+    if (c->storage == BTE_STORE_F32 && c->dim >= 2) {
         CU(c, launch_moment_rows(a, c->stream));
     } else {
         CU(c, launch_moment_only(a, c->storage, c->stream));
@@ -894,7 +892,6 @@ extern "C" bte_status bte_step(bte_ctx *c, int nsteps) {
     if (c->peer) return fail(c, BTE_ESTATE, "the context is coupled at an interface: it steps through bte_step_pair");
     // after synthetic iterations the step starts from the state's own T_L (Eq. BTE_get_e0)
     if (c->tl_corrected && nsteps > 0) TRY(refresh_moments(c));
-    if (nsteps > 0) c->fresh = false;
     if (c->persist) return nsteps > 0 ? step_persistent(c, nsteps) : BTE_OK;
     int s = 0;
     if (nsteps >= 2 * kGraphSteps && graph_eligible(c)) {
@@ -974,7 +971,6 @@ static cudaError_t launch_forward(bte_ctx *c, const StepArgs &a, cudaStream_t st
 }
 
 static bte_status step_one(bte_ctx *c, cudaStream_t strm) {
-    c->fresh = false;
     {
         StepArgs a = make_args(c);
         a.amp = (float)amplitude_at(c, c->step);
@@ -1496,12 +1492,17 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
     if (c->peer) return fail(c, BTE_ESTATE, "the context is coupled at an interface (no adjoint of the pair)");
     for (long long i = 0; i < c->ncell; ++i)
         if (!std::isfinite(probe[i])) return fail(c, BTE_EINVAL, "probe holds a non-finite value at cell %lld", i);
+    if (c->tl_corrected) TRY(refresh_moments(c));
+    // Where bte_step streams, its own steps lead to the end state (they cost less than a tenth of the call).
+    // Grids of a few cells have one trajectory, bte_step's: on them the two are equally far from 64 bits (18 runs
+    // a grid of 4 to 27 cells: dJ/dlog tau 0.5 to 1.6e-5 in the median by either, up to 5e-4).
+    constexpr long long kFewCells = 32;
+    const bool replay = c->streamed && c->ncell >= kFewCells;
     struct Plain {
         bte_ctx *c;
         ~Plain() { c->plain = false; }
     } plain{c};
-    c->plain = c->limiter == BTE_LIM_MINMOD && c->storage == BTE_STORE_F32 && c->dim >= 2;
-    if (c->tl_corrected || (c->plain && c->fresh)) TRY(refresh_moments(c));
+    c->plain = replay;
     const long long nc = c->ncell, nel = c->nelem;
     int K = ckpt_every > 0 ? ckpt_every : std::max(1, (int)std::ceil(std::sqrt((double)std::max(nsteps, 1))));
     K = std::max(1, std::min(K, std::max(nsteps, 1)));
@@ -1544,7 +1545,7 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
         if ((K2 > 1 || &s != &L2[0]) && !w.snap(s)) return fail(c, BTE_ENOMEM, "adjoint checkpoints do not fit in device memory");
     for (auto &s : L3)
         if (!w.snap(s)) return fail(c, BTE_ENOMEM, "adjoint checkpoints do not fit in device memory");
-    if (!w.snap(fin)) return fail(c, BTE_ENOMEM, "adjoint checkpoints do not fit in device memory");
+    if (!replay && !w.snap(fin)) return fail(c, BTE_ENOMEM, "adjoint checkpoints do not fit in device memory");
     // tiled adjoint: segment partials, wall corrections, block partials of sum mu T_L
     float *Pm = nullptr, *Pq = nullptr, *Ps = nullptr, *corr[3] = {nullptr, nullptr, nullptr};
     double *mtp = nullptr;
@@ -1666,7 +1667,7 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
             }
             TRY(timed_steps(n - keep + 1));
         }
-        TRY(snap_save(c, fin, w.ediff_bytes));
+        if (!replay) TRY(snap_save(c, fin, w.ediff_bytes));
         // J = sum p T_L^N and lambda^N
         {
             std::vector<float> tl(nc);
@@ -1717,7 +1718,13 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
                 for (int m = m1 - 1; m >= m0; --m) TRY(adj_step(L3[m - m0]));
             }
         }
-        TRY(snap_restore(c, fin, w.ediff_bytes));
+        if (!replay) {
+            TRY(snap_restore(c, fin, w.ediff_bytes));
+        } else if (nsteps > 0) {
+            TRY(snap_restore(c, L1[0], w.ediff_bytes));
+            c->plain = false;
+            TRY(timed_steps(nsteps));
+        }
         if (dJ_dQ) CU(c, cudaMemcpyAsync(dJ_dQ, gQ, nc * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         if (dJ_dlogtau) CU(c, cudaMemcpyAsync(dJ_dlogtau, gt, c->nb * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         CU(c, cudaStreamSynchronize(c->stream));

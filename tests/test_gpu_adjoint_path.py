@@ -42,7 +42,10 @@ def test_rows_without_a_tiled_adjoint(dim, n, bc, kernel):
                                       (2, (128, 13, 1), [PER, PER, SPE, DIF, PER, PER]),
                                       (2, (256, 6, 1), [DIF, SPE, PER, PER, PER, PER]),
                                       (3, (128, 5, 6), [ISO, DIF, SPE, SPE, PER, PER]),
-                                      (3, (128, 10, 7), [SPE, SPE, PER, PER, DIF, ISO])])
+                                      (3, (128, 10, 7), [SPE, SPE, PER, PER, DIF, ISO]),
+                                      # 3-D rows below 112 cells: bte_step streams by default
+                                      (3, (96, 10, 7), [SPE, SPE, PER, PER, DIF, ISO]),
+                                      (3, (80, 6, 5), [DIF, ISO, SPE, SPE, PER, PER])])
 def test_default_gradients_are_the_tiled_ones(dim, n, bc, limiter, storage):
     out = []
     for kernel in (0, 2):
@@ -70,3 +73,32 @@ def test_16bit_wall_pass_rounds_each_operation(dim, limiter, storage):
     cfg, P, ctx, Q, amps, dT0, p = _setup(dim, n, bc, limiter, 2, 6, storage=storage)
     _, _, gt = _gpu_adjoint(ctx, Q, amps, dT0, p, 6, ckpt=2)
     assert tuple(float(x).hex() for x in gt) == WALL_BITS[dim, limiter, storage]
+
+
+@pytest.mark.parametrize("limiter", [0, 1, 2])
+@pytest.mark.parametrize("dim,n,bc", [(2, (128, 9, 1), [SPE, DIF, ISO, DIF, PER, PER]),
+                                      (2, (37, 21, 1), [DIF, SPE, ISO, DIF, PER, PER]),
+                                      (3, (64, 6, 5), [SPE, ISO, PER, PER, DIF, SPE]),
+                                      (3, (13, 5, 4), [SPE, ISO, DIF, DIF, DIF, SPE])])
+def test_end_state_is_that_of_the_steps(dim, n, bc, limiter):
+    """By default, streamed or not: the state, T_L and the wall values (one more step) of bte_step, bit for
+    bit; nothing changes in a call of no steps; a repeated call gives the same gradients."""
+    from paper_2306_14181_gb300 import bte
+    out = []
+    for adjoint in (True, False):
+        cfg, P, ctx, Q, amps, dT0, p = _setup(dim, n, bc, limiter, 0, 7)
+        if adjoint:
+            first = _gpu_adjoint(ctx, Q, amps, dT0, p, 7, ckpt=3)
+            again = _gpu_adjoint(ctx, Q, amps, dT0, p, 7, ckpt=3)
+            assert first[0] == again[0] and np.array_equal(first[2], again[2])
+        else:
+            bte.bte_init_temperature(ctx, dT0.reshape(-1))
+            bte.bte_set_source(ctx, Q, amps)
+            bte.bte_step(ctx, 7)
+        end = [bte.bte_get_state(ctx).copy(), bte.bte_lattice_temperature(ctx).copy()]
+        J, _, _ = bte.bte_adjoint(ctx, 0, p, 0)
+        assert abs(J - float(np.sum(p.reshape(-1) * end[1].astype(np.float64)))) <= 1e-12 * abs(J)
+        bte.bte_step(ctx, 1)
+        end.append(bte.bte_get_state(ctx).copy())
+        out.append(end)
+    assert all(np.array_equal(x, y) for x, y in zip(*out))
