@@ -481,7 +481,7 @@ enum { kMomGeneral = 0, kMomOctant = 1, kMomAxis = 2 };
 
 __device__ __forceinline__ double widen(float f) {
     const uint32_t u = __float_as_uint(f), m = u & 0x7fffffffu;
-    if (m != 0u && m < 0x00800000u) return (double)f;  // a subnormal
+    if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)f;  // a subnormal, an infinity or a NaN
     const uint32_t hi = m == 0u ? u : ((u & 0x80000000u) | ((m >> 3) + 0x38000000u));
     return __hiloint2double((int)hi, (int)(u << 29));
 }
