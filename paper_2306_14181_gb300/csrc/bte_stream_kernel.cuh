@@ -37,7 +37,7 @@ namespace bte {
 namespace stream {
 
 constexpr int kThreads = 256;
-constexpr float kVaTiny = 1e-30f;
+constexpr float kVaTiny = 0x1p-125f;
 
 __device__ __forceinline__ float rcp_approx(float x) {
     float r;
@@ -48,8 +48,9 @@ __device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f), a); }
 
 // The limited slope L(a, b) of the upwind and downwind differences a, b; a face's value is e_m + L/2.
-// Van Albada: max(ab, 0) (a + b) / (a^2 + b^2 + 1e-30) with the approximate reciprocal of a denominator
-// that is always a normal number.
+// Van Albada: max(ab, 0) (a + b) / (a^2 + b^2 + 2^-125) with the approximate reciprocal of a denominator
+// that is always a normal number; the constant is below the last bit of the squares wherever the products of
+// the numerator are normal numbers, so slopes are limited alike in any units.
 template <int LIM> __device__ __forceinline__ float slope(float a, float b);
 template <> __device__ __forceinline__ float slope<kLimFirst>(float, float) { return 0.f; }
 template <> __device__ __forceinline__ float slope<kLimMinmod>(float a, float b) {
