@@ -418,12 +418,17 @@ cudaError_t launch_persist_1d(const StepArgs &a, int limiter, int nsteps, const 
                                                                                        : k_persist_1d<kLimVanAlbada>;
     cudaError_t err;
     const int nd = a.nd, n = a.n[0], nb = a.nb;
-    // as many threads as share the items (four cells each) evenly, at least one a cell for the sums
+    // As many threads as share the items (four cells each) evenly, at least one a cell for the sums, and a warp for
+    // each wall task as far as there are tasks for 16 warps: short rows have more tasks than cells.  Us a step by
+    // k_persist_1d / without that / with it: 5 cells, 100 x 8 2.71 / 3.27 / 2.30; 2 cells, 40 x 64 4.31 / 5.08 / 3.00.
+    // Long rows take all the threads there are: 600 cells, 1 x 8 5.1 / 5.9 / 4.7; 700 5.6 / 6.0 / 5.0.
     auto threads = [=](int C) {
-        const long long nit = (long long)((nb + C - 1) / C) * nd * ((n + 3) / 4);
+        const long long nbl = (nb + C - 1) / C, nit = nbl * nd * ((n + 3) / 4), tasks = 2 * nbl + (2 * nbl * nd + 31) / 32;
         const long long rounds = (nit + 1023) / 1024;
+        if (n > 512 && rounds > 1) return 1024;
         long long t = (nit + rounds - 1) / rounds;
         if (t < n) t = n;
+        if (t < 32 * tasks) t = tasks < 16 ? 32 * tasks : (t < 512 ? 512 : t);
         if (t < 128) t = 128;
         t = (t + 31) / 32 * 32;
         return t > 1024 ? 1024 : (int)t;
