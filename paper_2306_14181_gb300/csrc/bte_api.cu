@@ -953,10 +953,12 @@ extern "C" bte_status bte_interface(bte_ctx *a, int wa, bte_ctx *b, int wb, cons
     return iface_mix(a);
 }
 
-// The split 1-D step (update and sums apart) where few bands leave the generic step too few blocks; its sums
-// take the bands one after another.  Us a step, generic / split: 1000 cells, 1 x 512 20 / 7.5; 292 cells, 12 x
+// The split 1-D step (update and sums apart) where few bands of few cells leave the generic step too few blocks (up
+// to 3 an SM, each 8 cells by 32 groups of directions); it reads the state once more, and its sums take the bands
+// one after another.  Us a step, generic / split: 1000 cells, 1 x 512 26.7 / 10.0; 3000, 1 x 64 7.5 / 7.4; 1500, 2 x
+// 256 15.7 / 11.8; beyond the line 4000, 1 x 64 8.1 / 8.2; 3000, 2 x 64 8.9 / 10.8; 20000, 1 x 64 19 / 25; 292, 12 x
 // 16 6.9 / 15.2.
-static bool split_1d(const bte_ctx *c) { return c->dim == 1 && c->nb <= 2; }
+static bool split_1d(const bte_ctx *c) { return c->dim == 1 && c->nb <= 2 && c->ncell * c->nb <= 3 * 8 * 152; }
 
 // The forward step's main kernel by the context's plan.
 static cudaError_t launch_forward(bte_ctx *c, const StepArgs &a, cudaStream_t strm) {
