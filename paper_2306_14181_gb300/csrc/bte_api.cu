@@ -405,6 +405,11 @@ static bte_status prof_event(bte_ctx *c, cudaEvent_t *out) {
     return BTE_OK;
 }
 
+// Grids of fewer cells stream whatever the sizes say, and the adjoint differentiates that trajectory: its
+// gradients and those of the generic steps are equally far from 64 bits there (18 runs a grid of 4 to 27 cells:
+// dJ/dlog tau 0.5 to 1.6e-5 in the median by either, up to 5e-4), and a test bound holds the streamed ones.
+constexpr long long kFewCells = 32;
+
 // ------------------------------------------------------------------------------------------
 // ABI
 // ------------------------------------------------------------------------------------------
@@ -569,7 +574,16 @@ extern "C" bte_status bte_create(const bte_grid *grid, const bte_bands *bands, c
     // 1577, of 96 1733 / 1586, of 64 1521 / 1122; 32^2 x 16, 40 x 96 924 / 421; in 2-D 256^2, 20 x 128 318 / 442,
     // 128^2, 20 x 64 69 / 80, rows of 96 166 / 230, of 64 156 / 175, 200^2 296 / 284.
     const bool tiled_faster = c->tiled && (c->dim == 2 || (c->plan.nx == 128 && c->n[0] >= 112));
-    if (!c->persist && !tiled_faster && !(c->tiled && c->kernel == BTE_KERNEL_TILED)) {
+    // Grids the tiled kernel does not take run the generic one where they are small: it has a thread a (cell, band)
+    // and group of directions, the streaming kernel a longer chain of latencies, and rows of partials to add.  The
+    // line was drawn through 300 grids of 100 to 40000 cells, 1 to 40 bands, 8 to 128 directions; below it
+    // streaming took up to 4 times as long, above it it is at most 4 % slower.  Us a step, generic / streaming:
+    // 17 x 16, 40 x 128 32 / 62; 34 x 33, 4 x 128 16 / 26; 79 x 32, 2 x 128 14.0 / 16.6; 61 x 58, 2 x 96 21.1 / 15.9;
+    // 13 x 12 x 11, 10 x 32 20.9 / 30.0; 13 x 12 x 12, 20 x 128 61.8 / 64.6; 19 x 14 x 14, 11 x 48 40.5 / 28.2; few
+    // directions, 91 x 163, 1 x 8 7.1 / 9.5.  (Fewer than kFewCells: see there.)
+    const double dirs = std::min(c->nd, 32) / 32.0, size = (double)c->ncell * c->ncell * c->nb * dirs * dirs;
+    const bool generic_faster = !c->tiled && c->ncell >= kFewCells && size < (c->dim == 2 ? 2.5e7 : 1.2e8);
+    if (!c->persist && !tiled_faster && !generic_faster && !(c->tiled && c->kernel == BTE_KERNEL_TILED)) {
         std::string why;  // not applicable: the tiled or the generic kernel
         c->streamed = stream_plan(c->dim, c->n, c->nb, c->nd, c->s.data(), c->bc, c->jump, c->storage, c->limiter,
                                   c->splan, why);
@@ -1496,9 +1510,6 @@ extern "C" bte_status bte_adjoint(bte_ctx *c, int nsteps, int ckpt_every, const 
         if (!std::isfinite(probe[i])) return fail(c, BTE_EINVAL, "probe holds a non-finite value at cell %lld", i);
     if (c->tl_corrected) TRY(refresh_moments(c));
     // Where bte_step streams, its own steps lead to the end state (they cost less than a tenth of the call).
-    // Grids of a few cells have one trajectory, bte_step's: on them the two are equally far from 64 bits (18 runs
-    // a grid of 4 to 27 cells: dJ/dlog tau 0.5 to 1.6e-5 in the median by either, up to 5e-4).
-    constexpr long long kFewCells = 32;
     const bool replay = c->streamed && c->ncell >= kFewCells;
     struct Plain {
         bte_ctx *c;
