@@ -20,9 +20,12 @@
 // lane only ever reads its own stores.
 //
 // Bound by latency along a row and by the memory of the 33 warps an SM that the hot spot's 5120 planes
-// give: the next row's values are loaded (16 bytes a lane where rows allow) before this row's scan.
+// give: the next row's (longer rows: the next chunk's) own values are loaded, 16 bytes a lane where rows allow,
+// before this row's scan, and a row's z values with them.
 // An iteration on 256^2, 40 x 128: 2.41 -> 1.54 ms with this and k_moment_rows (the sweep alone was 1.11
-// ms with the y term read back and no loads ahead).
+// ms with the y term read back and no loads ahead).  Few planes, us an iteration without the loads ahead of long
+// rows and of the z values / with them: 20001 cells, 2 x 64 216 / 140; 130 x 16 x 16, 3 x 48 522 / 342, 20 x 96 1102 /
+// 878; 100^2, 1 x 8 93 / 79.
 #include <cuda_runtime.h>
 
 #include "bte_internal.h"
@@ -34,10 +37,11 @@ constexpr int kSweepWarps = 4;
 constexpr int kCellsPerLane = 4;
 
 // Chunks of a row held in registers: rows of up to CH * 128 cells (CH = 0: any length, the y term read
-// back like the z term).  VEC: rows are multiples of four cells, which move 16 bytes a lane.
-template <int CH, bool VEC>
-__global__ void __launch_bounds__(kSweepWarps * 32, 9) k_sis_sweep(const StepArgs a, const float *__restrict__ e_in,
-                                                                    float *e_io) {
+// back like the z term).  VEC: rows are multiples of four cells, which move 16 bytes a lane.  Z: 3-D, whose z values
+// take registers of their own, on their way together with the next loads.
+template <int CH, bool VEC, bool Z>
+__global__ void __launch_bounds__(kSweepWarps * 32, Z ? 6 : 9) k_sis_sweep(const StepArgs a, const float *__restrict__ e_in,
+                                                                           float *e_io) {
     const int lane = threadIdx.x & 31;
     const long long plane = (long long)blockIdx.x * kSweepWarps + (threadIdx.x >> 5);
     if (plane >= (long long)a.nb * a.nd) return;
@@ -75,72 +79,68 @@ __global__ void __launch_bounds__(kSweepWarps * 32, 9) k_sis_sweep(const StepArg
                 }
         }
     };
-    float no[NC][V], ni[NC][V], dp[NC][V];  // the next row's values; De of the row upwind in y
+    // the next chunks' values; De of the row upwind in y (CH = 0: its stored values dp and yi)
+    float no[NC][V], ni[NC][V], dp[NC][V], yi[V];
     #pragma unroll
     for (int c = 0; c < NC; ++c)
         #pragma unroll
-        for (int v = 0; v < V; ++v) no[c][v] = ni[c][v] = dp[c][v] = 0.f;
+        for (int v = 0; v < V; ++v) no[c][v] = ni[c][v] = dp[c][v] = yi[v] = 0.f;
     auto row_of = [&](int uz, int uy) {
         return ((long long)(sz > 0 ? uz : nz - 1 - uz) * ny + (sy > 0 ? uy : ny - 1 - uy)) * nx;
     };
-    if constexpr (CH > 0) {
-        #pragma unroll
-        for (int c = 0; c < NC; ++c) load(row_of(0, 0), c * 32 * V, no[c], ni[c]);
-    }
+    #pragma unroll
+    for (int c = 0; c < NC; ++c) load(row_of(0, 0), c * 32 * V, no[c], ni[c]);
     for (int uz = 0; uz < nz; ++uz) {
         for (int uy = 0; uy < ny; ++uy) {
             const long long row = row_of(uz, uy);
             float carry = 0.f;  // De of the cell before the chunk (0 at the upwind wall)
             const int nch = CH > 0 ? CH : (nx + 32 * V - 1) / (32 * V);
+            const int my = uy + 1 < ny ? uy + 1 : 0, mz = uy + 1 < ny ? uz : uz + 1;  // the next row
             float av[NC][V], vi[NC][V];
-            if constexpr (CH > 0) {
-                // right-hand sides of the row, then the next row's loads
+            // right-hand sides of the NC chunks at c0, their z term in step with the next chunks' loads
+            auto rhs = [&](int c0) {
+                float zo[NC][V], zi[NC][V];
+                if constexpr (Z) {
+                    if (uz > 0) {
+                        #pragma unroll
+                        for (int c = 0; c < NC; ++c) load(row - dzg, (c0 + c) * 32 * V, zo[c], zi[c]);
+                    }
+                }
+                if constexpr (CH == 0) {
+                    if (uy > 0) load(row - dyg, c0 * 32 * V, dp[0], yi);
+                }
                 #pragma unroll
                 for (int c = 0; c < NC; ++c)
                     #pragma unroll
                     for (int v = 0; v < V; ++v) {
                         vi[c][v] = ni[c][v];
-                        float r = no[c][v] - ni[c][v];  // dt R
-                        if (uy > 0) r = fmaf(nuy, dp[c][v], r);
-                        av[c][v] = r;
+                        av[c][v] = no[c][v] - ni[c][v];  // dt R
                     }
-                const int my = uy + 1 < ny ? uy + 1 : 0, mz = uy + 1 < ny ? uz : uz + 1;
-                if (mz < nz) {
+                const bool last = c0 + NC >= nch;
+                if (!last || mz < nz) {
                     #pragma unroll
-                    for (int c = 0; c < NC; ++c) load(row_of(mz, my), c * 32 * V, no[c], ni[c]);
+                    for (int c = 0; c < NC; ++c) load(last ? row_of(mz, my) : row, last ? c * 32 * V : (c0 + 1) * 32 * V, no[c], ni[c]);
                 }
-            }
-            #pragma unroll
-            for (int c = 0; c < nch; ++c) {
-                constexpr int kOne = 0;
-                const int q = CH > 0 ? c : kOne;
-                const int u = c * 32 * V + lane * V;
-                if constexpr (CH == 0) {
-                    float vo[V] = {0.f, 0.f, 0.f, 0.f};
-                    #pragma unroll
-                    for (int v = 0; v < V; ++v) vi[0][v] = 0.f;
-                    load(row, c * 32 * V, vo, vi[0]);
+                #pragma unroll
+                for (int c = 0; c < NC; ++c)
                     #pragma unroll
                     for (int v = 0; v < V; ++v) {
-                        float r = vo[v] - vi[0][v];
-                        if (uy > 0 && u + v < nx) {
-                            const long long i = row + xof(u + v) - dyg;
-                            r = fmaf(nuy, eo[i] - ei[i], r);
-                        }
-                        av[0][v] = r;
+                        if (uy > 0) av[c][v] = fmaf(nuy, CH > 0 ? dp[c][v] : dp[c][v] - yi[v], av[c][v]);
+                        if (Z && uz > 0) av[c][v] = fmaf(nuz, zo[c][v] - zi[c][v], av[c][v]);
                     }
-                }
+            };
+            if constexpr (CH > 0) rhs(0);
+            #pragma unroll(NC)
+            for (int c = 0; c < nch; ++c) {
+                if constexpr (CH == 0) rhs(c);
+                const int q = CH > 0 ? c : 0;
+                const int u = c * 32 * V + lane * V;
                 // the lane's map De_out = A + B De_in over its cells of the row
                 float A = 0.f, B = 1.f;
                 #pragma unroll
                 for (int v = 0; v < V; ++v) {
                     const bool in = u + v < nx;
-                    float r = av[q][v];
-                    if (uz > 0 && in) {
-                        const long long i = row + xof(u + v) - dzg;
-                        r = fmaf(nuz, eo[i] - ei[i], r);
-                    }
-                    av[q][v] = r * inv;
+                    av[q][v] *= inv;
                     A = in ? fmaf(b, A, av[q][v]) : A;
                     B = in ? B * b : B;
                 }
@@ -181,12 +181,12 @@ __global__ void __launch_bounds__(kSweepWarps * 32, 9) k_sis_sweep(const StepArg
     }
 }
 
-template <bool VEC>
+template <bool VEC, bool Z>
 void launch_sweep(const StepArgs &a, const float *e_in, float *e_io, unsigned blocks, cudaStream_t s) {
     const int chunks = (a.n[0] + 127) / 128;
-    if (chunks == 1) k_sis_sweep<1, VEC><<<blocks, kSweepWarps * 32, 0, s>>>(a, e_in, e_io);
-    else if (chunks == 2) k_sis_sweep<2, VEC><<<blocks, kSweepWarps * 32, 0, s>>>(a, e_in, e_io);
-    else k_sis_sweep<0, VEC><<<blocks, kSweepWarps * 32, 0, s>>>(a, e_in, e_io);
+    if (chunks == 1) k_sis_sweep<1, VEC, Z><<<blocks, kSweepWarps * 32, 0, s>>>(a, e_in, e_io);
+    else if (chunks == 2) k_sis_sweep<2, VEC, Z><<<blocks, kSweepWarps * 32, 0, s>>>(a, e_in, e_io);
+    else k_sis_sweep<0, VEC, Z><<<blocks, kSweepWarps * 32, 0, s>>>(a, e_in, e_io);
 }
 
 }  // namespace
@@ -194,8 +194,14 @@ void launch_sweep(const StepArgs &a, const float *e_in, float *e_io, unsigned bl
 cudaError_t launch_sis_sweep(const StepArgs &a, const float *e_in, float *e_io, cudaStream_t s) {
     const long long planes = (long long)a.nb * a.nd;
     const unsigned blocks = (unsigned)((planes + kSweepWarps - 1) / kSweepWarps);
-    if (a.n[0] % kCellsPerLane == 0) launch_sweep<true>(a, e_in, e_io, blocks, s);
-    else launch_sweep<false>(a, e_in, e_io, blocks, s);
+    const bool vec = a.n[0] % kCellsPerLane == 0;
+    if (a.n[2] > 1) {
+        if (vec) launch_sweep<true, true>(a, e_in, e_io, blocks, s);
+        else launch_sweep<false, true>(a, e_in, e_io, blocks, s);
+    } else {
+        if (vec) launch_sweep<true, false>(a, e_in, e_io, blocks, s);
+        else launch_sweep<false, false>(a, e_in, e_io, blocks, s);
+    }
     return cudaGetLastError();
 }
 
