@@ -46,7 +46,9 @@ __global__ void __launch_bounds__(1024, 1) k_persist_1d(const StepArgs a, int ns
     const int n = a.n[0], nd = a.nd;
     const int nbl = (a.nb - rank + C - 1) / C;  // bands of this CTA: rank, rank + C, ...
     const int npl = nbl * nd, nel = npl * n;
-    float *e0 = sm, *e1 = sm + nel, *tl = e1 + nel;
+    // laid out for rank 0's bands (the most): peers read one another's part at the same place
+    const int nelm = (a.nb + C - 1) / C * nd * n;
+    float *e0 = sm, *e1 = sm + nelm, *tl = e1 + nelm;
     float *part = tl + n;  // [2][n] this CTA's share of the T_L numerator, read by the cluster
     float *ed = part + 2 * n;  // [2][nbl] diffuse-wall values of this CTA's bands
     float *pnu = ed + 2 * nbl, *pwm = pnu + npl, *pdt = pwm + npl, *pck = pdt + npl, *psr = pck + npl;
