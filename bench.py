@@ -419,7 +419,7 @@ def roofline_of(info, steps, fwd_ms, nfwd, fin_ms, nfin, peak, peak_kind, traffi
     if persistent:
         # the state stays in shared memory: report the step time, not a DRAM fraction
         r["us_per_step"] = fwd_avg_s * 1e6 / steps_per_launch
-        r["note"] = "one single-CTA launch per bte_step call; the state never leaves shared memory"
+        r["note"] = "one cluster launch per bte_step call; the state never leaves shared memory"
         r["finalize_ms"] = 0.0
     return r
 
@@ -454,8 +454,8 @@ def adjoint_record(ctx, cfg, info, fwd_step_ms, nadj, kck, Q, amps, peak):
 # Sub-records measured in the same run after the headline, one context at a time: (workload,
 # storage, T_scale, timed forward steps, adjoint steps or None, checkpoint spacing, kernel).
 # The 3-D adjoint runs 100 of its 1000 steps (checkpoints every 50) to keep the run within
-# minutes.  The hot spot also runs on the generic kernel (one thread per cell and band), the
-# path grids of any shape take.
+# minutes.  The hot spot also runs with the explicit generic choice, the path of grids the tiled
+# kernel does not take (at this size the register-streaming kernel).
 SUB_RECORDS = [
     ("laser_3d", "f16", 1.0, 30, None, None, "auto"),
     ("hotspot_2d", "f32", 1.0, 100, None, None, "auto"),

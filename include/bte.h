@@ -98,11 +98,11 @@ enum {
     BTE_KERNEL_AUTO = 0,       /* persistent for small 1-D FP32 problems, else tiled where its shape
                                   limits allow, else generic; a grid that is tiled may still take its
                                   forward step on the register-streaming kernel where that is faster */
-    BTE_KERNEL_GENERIC = 1,    /* the kernels for grids of any shape: register-streaming (2-D and 3-D,
-                                  FP32 storage), else one thread per (cell, band) */
+    BTE_KERNEL_GENERIC = 1,    /* the kernels for grids of any shape: register-streaming (larger 2-D and
+                                  3-D grids, FP32 storage), else one thread per (cell, band) */
     BTE_KERNEL_TILED = 2,      /* shared-memory tiled kernel; BTE_EUNSUPPORTED if the grid does not fit */
-    BTE_KERNEL_PERSISTENT = 3  /* 1-D, FP32 storage, state in one CTA's shared memory for all the steps
-                                  of a bte_step call (two block barriers a step, one launch a call);
+    BTE_KERNEL_PERSISTENT = 3  /* 1-D, FP32 storage, a state that fits one CTA's shared memory: held by one
+                                  cluster for all the steps of a bte_step call (one launch a call);
                                   BTE_EUNSUPPORTED otherwise */
 };
 
@@ -174,8 +174,9 @@ typedef struct {
     long long nelem;        /* nbands * ndirs * ncell, the updates per step */
     size_t state_bytes;     /* nelem * element size; the size bte_get_state/bte_set_state take */
     int elem_bytes;         /* 4 (FP32) or 2 (16-bit) */
-    int storage, limiter, kernel; /* kernels used: BTE_KERNEL_GENERIC, _TILED (the tiled adjoint, and the
-                                     forward step unless the streaming kernel is faster) or _PERSISTENT */
+    int storage, limiter, kernel; /* kernels used: BTE_KERNEL_GENERIC, _TILED (the steps bte_adjoint
+                                     differentiates, and bte_step's unless the streaming kernel is faster) or
+                                     _PERSISTENT */
     double dt;
     double W;               /* sum_d w_d */
     long long step;         /* steps taken since bte_init_temperature / bte_set_state */

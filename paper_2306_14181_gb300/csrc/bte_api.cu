@@ -66,7 +66,7 @@ struct bte_ctx {
     // tiled-kernel plan
     TiledPlan plan;
     bool tiled = false;
-    // register-streaming plan (FP32, 2-D and 3-D): the forward step of the grids the tiled kernel does not
+    // register-streaming plan (FP32, 2-D and 3-D): the forward step of the larger grids the tiled kernel does not
     // take and of those it takes but steps slower; precedes `tiled`, which then keeps the adjoint
     StreamPlan splan;
     bool streamed = false;
@@ -74,7 +74,7 @@ struct bte_ctx {
     // bte_step streams.  dJ/dlog tau is a sum that cancels, and a last-bit change of the states moves it by up
     // to 1e-3 (minmod's gradient also jumps where two slopes are equal).
     bool plain = false;
-    // persistent single-CTA path (small 1-D FP32 problems): per-call source amplitudes
+    // persistent path, one cluster (small 1-D FP32 problems): per-call source amplitudes
     bool persist = false;
     float *d_amp = nullptr;
     size_t d_amp_n = 0;
@@ -807,7 +807,7 @@ extern "C" bte_status bte_set_source(bte_ctx *c, const float *Q, int on_device, 
     return BTE_OK;
 }
 
-// All nsteps steps in one persistent single-CTA launch (1-D FP32 states in shared memory).
+// All nsteps steps in one persistent launch of one cluster (1-D FP32 states in shared memory).
 static bte_status step_persistent(bte_ctx *c, int nsteps) {
     if ((size_t)nsteps > c->d_amp_n) {
         if (c->d_amp) cudaFree(c->d_amp);
@@ -1351,7 +1351,7 @@ extern "C" bte_status bte_get_info(const bte_ctx *c, bte_info *info) {
     info->W = c->W;
     info->step = c->step;
     info->device_bytes = c->device_bytes;
-    // forward + finalize passes (the tiled finalize adds one for walls that need ghost values)
+    // forward + finalize passes
     info->launches_per_step = c->persist ? 1 : 2;
     return BTE_OK;
 }

@@ -13,9 +13,10 @@
 namespace bte {
 
 // ------------------------------------------------------------------------------------------
-// Generic forward step: one thread per (cell, band), looping over the band's directions (2-D and 3-D
-// grids: 16-bit states the tiled kernel does not take, and planes too large for the streaming kernel's 32-bit
-// indices; other FP32 grids run bte_stream_kernel.cuh).
+// Generic forward step: one thread per (cell, band), looping over the band's directions.  Runs 1-D grids the
+// persistent and the split step do not take; 2-D and 3-D grids the tiled kernel does not take where the state has 16
+// bits, the grid is small or a plane too large for the streaming kernel's 32-bit indices; and, where bte_step
+// streams, the steps bte_adjoint differentiates.
 // Eq. (disretized_transientBTE) with the limited upwind face value of Sec. 4.1, in upwind
 // orientation: with sg = sign(nu_a) and u_j = e(i + j sg),
 //   e_out = u_0 + L(u_0 - u_-1, u_1 - u_0)/2,  e_in = u_-1 + L(u_-1 - u_-2, u_0 - u_-1)/2,

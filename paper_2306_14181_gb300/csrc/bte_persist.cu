@@ -410,8 +410,6 @@ static size_t persist_smem(const StepArgs &a, int C) {
     return (2 * npl * a.n[0] + 3 * (size_t)a.n[0] + 2 * nbl + 5 * npl) * sizeof(float);
 }
 
-size_t persist_1d_smem(const StepArgs &a) { return persist_smem(a, 1); }
-
 cudaError_t launch_persist_1d(const StepArgs &a, int limiter, int nsteps, const float *amps, float *e_io,
                               float *tl_out, float *ediff_out, cudaStream_t s) {
     using Kern = void (*)(const StepArgs, int, const float *, float *, float *, float *);

@@ -121,10 +121,8 @@ bool stream_plan(int dim, const int n[3], int nb, int nd, const double *s, const
     plan.nys = (n[1] + plan.kr - 1) / plan.kr;
     plan.nz = n[2];
     plan.G = (n[0] + 1) / 2;
-    for (int a = 0; a < dim; ++a) {
-        if (bc[2 * a] == kBcSpecular || bc[2 * a + 1] == kBcSpecular) plan.spec |= 1 << a;
+    for (int a = 0; a < dim; ++a)
         if (jump[a] != 0.0) plan.jump |= 1 << a;
-    }
     plan.E = std::min(plan.G, n[0] % 2 ? 3 : 2);  // the last group of an odd row overlaps the one before it
     const long long strips = (long long)plan.nys * plan.nz;
     if (strips * plan.G > INT_MAX) {
@@ -206,7 +204,6 @@ cudaError_t launch_step_stream(const StepArgs &a, const StreamPlan &plan, cudaSt
     p.nspecial = plan.nspecial;
     p.mixed = plan.mixed;
     for (int c = 0; c < 3; ++c) p.blocks[c] = plan.blocks[c];
-    p.spec = plan.spec;
     p.jump = plan.jump;
     const unsigned blocks = (unsigned)(plan.blocks[0] + plan.blocks[1] + plan.blocks[2]) * (unsigned)(a.nb * plan.nchunk);
     ((StreamKernel)plan.kernel)<<<blocks, kThreads, 0, s>>>(a, p);

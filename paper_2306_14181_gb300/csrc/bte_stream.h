@@ -1,4 +1,4 @@
-// Register-streaming forward kernel of the explicit DOM step for 2-D and 3-D grids of any shape
+// Register-streaming forward kernel of the explicit DOM step for 2-D and 3-D grids of any shape, FP32 states:
 // launch interface (the kernel is described in bte_stream_kernel.cuh).
 #pragma once
 
@@ -20,7 +20,7 @@ struct StreamArgs {
     int blocks[3];    // blocks a (band, part): groups next to an x wall, the other groups of the
                       // special strips, the rest
     int mixed;        // the slow blocks spread among the others, else first
-    int spec, jump;   // bit a: specular walls / a periodic temperature jump on axis a
+    int jump;         // bit a: a periodic temperature jump on axis a
 };
 
 struct StreamPlan {
@@ -28,7 +28,7 @@ struct StreamPlan {
     int dim = 0;
     int kr = 1, nchunk = 1;
     int nys = 1, nz = 1, G = 0, E = 0, nspecial = 0, mixed = 0, blocks[3] = {0, 0, 0};
-    int spec = 0, jump = 0;
+    int jump = 0;
     void *kernel = nullptr;
     int *dord = nullptr, *strips = nullptr;
     std::vector<int> h_dord, h_strips;

@@ -1,6 +1,7 @@
 // Register-streaming forward step of the explicit DOM scheme (arXiv 2306.14181, Sec. 4, Eq.
 // disretized_transientBTE) for 2-D and 3-D grids of any shape, any wall, with
-// FP32 states; included by the instantiation units bte_stream_<dim>d.cu.
+// FP32 states (small grids are faster on the generic kernel and run it); included by the instantiation
+// units bte_stream_<dim>d.cu.
 //
 // A thread owns two neighbouring cells of a row and KR rows, and loops over a part of one band's
 // directions.  Per direction it streams the rows from upwind to downwind straight from global memory:
